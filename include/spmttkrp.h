@@ -67,8 +67,9 @@ typedef struct {
                        kappa) is fixed when the plan is built                    */
   int nblk;         /* blocks per mode (warp blocks for variant 0, CTA blocks for
                        variant 1); 0 = size-based default                         */
-  int tile;         /* nonzeros per staged warp tile: 0 (= 128, halved while two
-                       CTAs per SM would not fit), 32, 64, 128 or 256             */
+  int tile;         /* nonzeros per staged warp tile: 0 (= 64, or 128 of 16 bytes;
+                       halved while two CTAs per SM would not fit), 32, 64, 128 or
+                       256; rounded to whole chunks of the lane groups            */
   size_t max_bytes; /* cap on the plan's device memory; 0 = no cap               */
   int checks;       /* 1 = synchronize and read the device error word after every
                        compute call (slow; for debugging)                         */
@@ -87,7 +88,7 @@ typedef struct {
                        0; otherwise form 0 runs): 7 warps per CTA compute and
                        the 8th stores the CTA's 960-nonzero write-order tiles
                        in destination order                                     */
-  int unroll;       /* nonzeros in flight per lane group in form 0: 0 (= 8), 4, 8 */
+  int unroll;       /* steps in flight per lane group in form 0, 3 modes: 0 (= 8), 4, 8 */
   int stages;       /* tiles per warp ring in form 0: 0 (= 2 for 32-byte and wider
                        nonzeros, 3 for 16-byte ones), 2, 3 or 4                   */
   int element_bytes;/* stride of a stored nonzero (N int32 indices + FP32 value):

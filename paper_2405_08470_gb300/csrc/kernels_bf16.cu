@@ -73,9 +73,20 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
     }
   }
   if (a.variant == 1) return launch_direct_bfloat16(a, c, s);
-  if (c.vec && c.VW == 4) {  // 8-byte lane slices (R <= 32): the FP32 kernel's lane shape
+  if (c.VW < 4 && narrow_built(a, c)) return launch_narrow_bf16(a, c, s);
+  if (c.vec && c.VW == 4) {  // 8-byte lane slices: the FP32 kernel's lane shape
     switch (a.nmodes) {
       case 3:
+        if (c.L == 1) {  // one-lane groups: 32 runs per warp, 4 nonzeros of each per tile
+          switch (a.mode + (a.es == 32 ? 0 : 3)) {
+            case 0: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 0, 32>(a, c.L, s);
+            case 1: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 1, 32>(a, c.L, s);
+            case 2: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 2, 32>(a, c.L, s);
+            case 3: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 0, 16>(a, c.L, s);
+            case 4: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 1, 16>(a, c.L, s);
+            default: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 2, 16>(a, c.L, s);
+          }
+        }
         if (a.es == 32) {
           switch (a.mode) {
             case 0: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 0, 32>(a, c.L, s);
@@ -84,17 +95,17 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
           }
         }
         switch (a.mode) {
-          case 0: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 0>(a, c.L, s);
-          case 1: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 1>(a, c.L, s);
-          default: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 2>(a, c.L, s);
+          case 0: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 0, 16>(a, c.L, s);
+          case 1: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 1, 16>(a, c.L, s);
+          default: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 8, 2, 16>(a, c.L, s);
         }
-      case 4: return launch_warp_kernel<4, __nv_bfloat16, 4, 1, 4>(a, c.L, s);
-      case 5: return launch_warp_kernel<5, __nv_bfloat16, 4, 1, 4>(a, c.L, s);
-      case 6: return launch_warp_kernel<6, __nv_bfloat16, 4, 1, 4>(a, c.L, s);
+      case 4: return launch_modes<4, __nv_bfloat16, 4, 4>(a, c.L, s);
+      case 5: return launch_modes<5, __nv_bfloat16, 4, 4>(a, c.L, s);
+      case 6: return launch_modes<6, __nv_bfloat16, 4, 4>(a, c.L, s);
       default: return launch_warp_kernel<0, __nv_bfloat16, 4, 1, 4>(a, c.L, s);
     }
   }
-  if (c.vec) {
+  if (c.vec && c.VW == 8) {
     switch (a.nmodes) {
       case 3:
         if (a.es == 32 && a.unroll == 4) {  // 32-byte nonzeros, 4 in flight, 3 CTAs/SM
@@ -113,22 +124,23 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
         }
         if (a.unroll == 4) {
           switch (a.mode) {
-            case 0: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 4, 0>(a, c.L, s);
-            case 1: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 4, 1>(a, c.L, s);
-            default: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 4, 2>(a, c.L, s);
+            case 0: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 4, 0, 16>(a, c.L, s);
+            case 1: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 4, 1, 16>(a, c.L, s);
+            default: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 4, 2, 16>(a, c.L, s);
           }
         }
         switch (a.mode) {
-          case 0: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 8, 0>(a, c.L, s);
-          case 1: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 8, 1>(a, c.L, s);
-          default: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 8, 2>(a, c.L, s);
+          case 0: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 8, 0, 16>(a, c.L, s);
+          case 1: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 8, 1, 16>(a, c.L, s);
+          default: return launch_warp_kernel<3, __nv_bfloat16, 8, 1, 8, 2, 16>(a, c.L, s);
         }
-      case 4: return launch_warp_kernel<4, __nv_bfloat16, 8, 1, 4>(a, c.L, s);
-      case 5: return launch_warp_kernel<5, __nv_bfloat16, 8, 1, 4>(a, c.L, s);
-      case 6: return launch_warp_kernel<6, __nv_bfloat16, 8, 1, 4>(a, c.L, s);
+      case 4: return launch_modes<4, __nv_bfloat16, 8, 4>(a, c.L, s);
+      case 5: return launch_modes<5, __nv_bfloat16, 8, 4>(a, c.L, s);
+      case 6: return launch_modes<6, __nv_bfloat16, 8, 2>(a, c.L, s);
       default: return launch_warp_kernel<0, __nv_bfloat16, 8, 1, 4>(a, c.L, s);
     }
   }
+  if (c.vec) return launch_warp_kernel<0, __nv_bfloat16, 2, 1, 4>(a, c.L, s);
   switch (c.RC) {
     case 1: return launch_warp_kernel<0, __nv_bfloat16, 1, 1, 4>(a, c.L, s);
     case 2: return launch_warp_kernel<0, __nv_bfloat16, 1, 2, 4>(a, c.L, s);

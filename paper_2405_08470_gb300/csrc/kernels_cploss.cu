@@ -168,10 +168,10 @@ __global__ void __launch_bounds__(256, 4) cp_fwd_batched_kernel(const uint8_t* _
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       float p[VW], x[VW];
-      Landing<T, VW, 1>::unpack(raw[u][0], p);
+      Piece<T, VW>::unpack(raw[u][0], p);
 #pragma unroll
       for (int k = 1; k < NT; ++k) {
-        Landing<T, VW, 1>::unpack(raw[u][k], x);
+        Piece<T, VW>::unpack(raw[u][k], x);
 #pragma unroll
         for (int j = 0; j < VW; ++j) p[j] *= x[j];
       }

@@ -50,10 +50,13 @@ int launch_mttkrp_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
     }
   }
   if (a.variant == 1) return launch_direct_float(a, c, s);
-  if (c.vec) {
+  if (c.VW < 4 && narrow_built(a, c)) return launch_narrow_f32(a, c, s);
+  if (c.vec && c.VW == 4) {
     switch (a.nmodes) {
       case 3:
-        if (a.es == 32 && a.unroll == 4) {  // 32-byte nonzeros, 4 in flight, 3 CTAs/SM
+        // 4 in flight and 3 CTAs per SM when asked for, and for one-lane groups, whose
+        // warps hold 32 runs (their tiles hold 4 nonzeros per run)
+        if (a.es == 32 && (a.unroll == 4 || c.L == 1)) {
           switch (a.mode) {
             case 0: return launch_warp_kernel<3, float, 4, 1, 4, 0, 32>(a, c.L, s);
             case 1: return launch_warp_kernel<3, float, 4, 1, 4, 1, 32>(a, c.L, s);
@@ -67,24 +70,25 @@ int launch_mttkrp_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
             default: return launch_warp_kernel<3, float, 4, 1, 8, 2, 32>(a, c.L, s);
           }
         }
-        if (a.unroll == 4) {
+        if (a.unroll == 4 || c.L == 1) {
           switch (a.mode) {
-            case 0: return launch_warp_kernel<3, float, 4, 1, 4, 0>(a, c.L, s);
-            case 1: return launch_warp_kernel<3, float, 4, 1, 4, 1>(a, c.L, s);
-            default: return launch_warp_kernel<3, float, 4, 1, 4, 2>(a, c.L, s);
+            case 0: return launch_warp_kernel<3, float, 4, 1, 4, 0, 16>(a, c.L, s);
+            case 1: return launch_warp_kernel<3, float, 4, 1, 4, 1, 16>(a, c.L, s);
+            default: return launch_warp_kernel<3, float, 4, 1, 4, 2, 16>(a, c.L, s);
           }
         }
         switch (a.mode) {
-          case 0: return launch_warp_kernel<3, float, 4, 1, 8, 0>(a, c.L, s);
-          case 1: return launch_warp_kernel<3, float, 4, 1, 8, 1>(a, c.L, s);
-          default: return launch_warp_kernel<3, float, 4, 1, 8, 2>(a, c.L, s);
+          case 0: return launch_warp_kernel<3, float, 4, 1, 8, 0, 16>(a, c.L, s);
+          case 1: return launch_warp_kernel<3, float, 4, 1, 8, 1, 16>(a, c.L, s);
+          default: return launch_warp_kernel<3, float, 4, 1, 8, 2, 16>(a, c.L, s);
         }
-      case 4: return launch_warp_kernel<4, float, 4, 1, 4>(a, c.L, s);
-      case 5: return launch_warp_kernel<5, float, 4, 1, 4>(a, c.L, s);
-      case 6: return launch_warp_kernel<6, float, 4, 1, 4>(a, c.L, s);
+      case 4: return launch_modes<4, float, 4, 4>(a, c.L, s);
+      case 5: return launch_modes<5, float, 4, 4>(a, c.L, s);
+      case 6: return launch_modes<6, float, 4, 2>(a, c.L, s);
       default: return launch_warp_kernel<0, float, 4, 1, 4>(a, c.L, s);
     }
   }
+  if (c.vec) return launch_warp_kernel<0, float, 2, 1, 4>(a, c.L, s);
   switch (c.RC) {
     case 1: return launch_warp_kernel<0, float, 1, 1, 4>(a, c.L, s);
     case 2: return launch_warp_kernel<0, float, 1, 2, 4>(a, c.L, s);

@@ -1,5 +1,9 @@
 // kernels_misc.cu - split-row fix-up, zero fill, remap-only pass, and the
 // dispatcher of the fused spMTTKRP + remap kernel.
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include "mttkrp_kernel.cuh"
 #include "mttkrp_tile.cuh"
 
@@ -12,20 +16,40 @@ int launch_mttkrp_tile(const MttkrpArgs& a, cudaStream_t s);
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 static LaneCfg cfg_for(const MttkrpArgs& a) {
-  bool al = aligned16(a.out);
+  uintptr_t all = 0;  // the factors' addresses, or'ed: its lowest set bit is their alignment
   for (int k = 0; k < a.nmodes; ++k)
-    if (k != a.mode) al = al && aligned16(a.factors[k]);
-  return lane_config(a.R, a.dtype, al, a.variant == 0 || a.variant == 3);  // form 0's lanes
+    if (k != a.mode || a.loss_part) all |= (uintptr_t)a.factors[k];
+  const size_t fa = all & 15u ? (size_t)(all & (~all + 1)) : 16;
+  const size_t oa = (uintptr_t)a.out & 15u ? (size_t)((uintptr_t)a.out & (~(uintptr_t)a.out + 1)) : 16;
+  if (a.variant == 1 || a.variant == 2) return lane_config(a.R, a.dtype, fa == 16 && oa == 16);
+  return warp_lane_config(a.R, a.dtype, fa, oa);
 }
 
 size_t mttkrp_smem_bytes(int es, int tile, int R, int dtype, int stages) {
   size_t m = 0;
-  for (bool al : {true, false}) {
-    const LaneCfg c = lane_config(R, dtype, al, true);
+  for (size_t al : {16, 8, 4}) {
+    const LaneCfg c = warp_lane_config(R, dtype, al, al);
     const int G = 32 / c.L;
-    m = std::max(m, (size_t)kWarps * warp_layout(es, warp_tile_for(tile, G), R, G, stages).total);
+    m = std::max(m, (size_t)kWarps * warp_layout(es, warp_tile_for(tile, G, 4), stages, true).total);
   }
   return m;
+}
+
+int resident_ctas(const void* kernel, size_t smem, int* ctas) {
+  static std::mutex mu;
+  static std::map<std::tuple<const void*, size_t, int>, int> known;
+  int dev = 0;
+  SPM_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  int& have = known[std::make_tuple(kernel, smem, dev)];
+  if (have == 0) {
+    int sms = 0, occ = 0;
+    SPM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    SPM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kThreads, smem));
+    have = std::max(1, occ) * sms;
+  }
+  *ctas = have;
+  return SPM_OK;
 }
 
 int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s) {
@@ -42,10 +66,12 @@ int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s) {
       return launch_mttkrp_tile(a, s);
     MttkrpArgs b = a;
     b.variant = 0;
+    c = cfg_for(b);
     return a.dtype == SPM_DTYPE_BF16 ? launch_mttkrp_bf16(b, c, s) : launch_mttkrp_f32(b, c, s);
   }
   if (a.variant == 3 &&
-      !(c.vec && a.nmodes == 3 && a.es == 32 && a.alpha_word && a.no_fill == 0 && a.elems_out)) {
+      !(c.vec && c.VW >= 4 && c.L > 1 && a.nmodes == 3 && a.es == 32 && a.alpha_word && a.no_fill == 0 &&
+        a.elems_out)) {
     // form 3 needs 32-byte 3-mode nonzeros with their ids and write orders, the
     // contiguous split, and a remap to do; otherwise form 0
     MttkrpArgs b = a;
@@ -212,19 +238,21 @@ int launch_scale_copy(const float* src, float* dst, int64_t n, const float* scal
   return e == cudaSuccess ? SPM_OK : cuda_fail(e, "scale_copy_kernel launch");
 }
 
-// 1/2 sum of n FP64 partials in a fixed order: thread t adds a contiguous chunk,
-// then the 256 chunk sums are added in a fixed tree; loss = that half-sum.
-__global__ void __launch_bounds__(256) loss_reduce_kernel(const double* __restrict__ part,
-                                                          int64_t n, float* __restrict__ loss,
-                                                          double* __restrict__ loss64) {
-  __shared__ double red[256];
-  const int64_t chunk = (n + 255) / 256;
-  const int64_t b = (int64_t)threadIdx.x * chunk, e = min(n, b + chunk);
+// 1/2 sum of n FP64 partials in a fixed order: thread t adds entries t, t + 1024, ...
+// (neighbouring threads read neighbouring entries, eight loads of each in flight: a
+// block's partial each, up to 150K of them, took 0.2 ms as 256 contiguous chunks), then
+// the threads' sums are added in a fixed tree; loss = that half-sum.
+constexpr int kLossThreads = 1024;
+__global__ void __launch_bounds__(kLossThreads) loss_reduce_kernel(
+    const double* __restrict__ part, int64_t n, float* __restrict__ loss,
+    double* __restrict__ loss64) {
+  __shared__ double red[kLossThreads];
   double acc = 0.0;
-  for (int64_t i = b; i < e; ++i) acc += part[i];
+#pragma unroll 8
+  for (int64_t i = threadIdx.x; i < n; i += kLossThreads) acc += part[i];
   red[threadIdx.x] = acc;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
+  for (int w = kLossThreads / 2; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();
   }
@@ -236,7 +264,7 @@ __global__ void __launch_bounds__(256) loss_reduce_kernel(const double* __restri
 
 int launch_loss_reduce(const double* part, int64_t n, float* loss, double* loss64,
                        cudaStream_t s) {
-  loss_reduce_kernel<<<1, 256, 0, s>>>(part, n, loss, loss64);
+  loss_reduce_kernel<<<1, kLossThreads, 0, s>>>(part, n, loss, loss64);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SPM_OK : cuda_fail(e, "loss_reduce_kernel launch");
 }

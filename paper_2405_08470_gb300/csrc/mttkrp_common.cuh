@@ -50,6 +50,26 @@ inline LaneCfg lane_config(int R, int dtype, bool aligned16, bool narrow_bf16 = 
   return c;
 }
 
+// Lanes of the warp-block form: the widest piece (values per lane and load) that
+// divides the rank, fits 32 lanes and suits the alignment of the factors and the
+// output, so that a rank that is no multiple of four still loads 8 bytes a lane (or 4,
+// or 2) with as many nonzeros per warp as its lanes allow.
+inline LaneCfg warp_lane_config(int R, int dtype, size_t factor_align, size_t out_align) {
+  const size_t es = dtype == SPM_DTYPE_BF16 ? 2 : 4;
+  for (int vw : {8, 4, 2}) {
+    if (vw == 8 && (dtype != SPM_DTYPE_BF16 || R <= 32)) continue;  // narrow BF16: FP32's lanes
+    if (R % vw || R / vw > 32 || factor_align % (vw * es) || out_align % (vw >= 4 ? 16 : 4 * vw))
+      continue;
+    LaneCfg c;
+    c.vec = true;
+    c.VW = vw;
+    c.L = pow2ceil(R / vw);
+    c.RC = 1;
+    return c;
+  }
+  return lane_config(R, dtype, false);
+}
+
 // ------------------------------------------------------------ stored nonzeros
 
 // Index k of a stored nonzeros (plain: word k; packed: its bit field).
@@ -107,6 +127,16 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// 16-byte asynchronous copy global -> shared by one thread, and the wait for all of
+// the thread's copies.
+__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // 1D bulk async copy with an L2 cache policy (e.g. evict_first for streams).
 __device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32_t bytes,
                                               uint64_t* bar, uint64_t policy) {
@@ -158,7 +188,7 @@ __device__ __forceinline__ uint4 ld_nc_hint_v4(const void* ptr, uint64_t policy)
   return v;
 }
 
-// 8-byte read-only global load with an L2 cache policy, and with an L1 choice.
+// 8-byte read-only global load with an L2 cache policy.
 __device__ __forceinline__ uint2 ld_nc_hint_v2(const void* ptr, uint64_t policy) {
   uint2 v;
   asm volatile("ld.global.nc.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
@@ -166,16 +196,10 @@ __device__ __forceinline__ uint2 ld_nc_hint_v2(const void* ptr, uint64_t policy)
                : "l"(ptr), "l"(policy));
   return v;
 }
-__device__ __forceinline__ uint2 ld_nc_l1_v2(const void* ptr, uint64_t policy, bool keep) {
-  uint2 v;
-  if (keep)
-    asm volatile("ld.global.nc.L1::evict_last.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
-                 : "=r"(v.x), "=r"(v.y)
-                 : "l"(ptr), "l"(policy));
-  else
-    asm volatile("ld.global.nc.L1::evict_first.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
-                 : "=r"(v.x), "=r"(v.y)
-                 : "l"(ptr), "l"(policy));
+// 4-byte read-only global load with an L2 cache policy.
+__device__ __forceinline__ uint32_t ld_nc_hint_v1(const void* ptr, uint64_t policy) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(ptr), "l"(policy));
   return v;
 }
 

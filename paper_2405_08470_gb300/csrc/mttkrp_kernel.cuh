@@ -1,30 +1,50 @@
-// mttkrp_kernel.cuh - the fused mode-n spMTTKRP + dynamic remap kernel,
-// one warp per block of the split.
+// mttkrp_kernel.cuh - the fused mode-n spMTTKRP + dynamic remap kernel, a persistent
+// grid of warps taking small blocks of the split.
 //
-// Every warp owns one block [lo, hi) of the mode-n ordered working copy (the
-// paper's thread block over a tensor partition, Algorithm 4, shrunk to a warp
-// so that no CTA-wide synchronisation is ever needed).  The warp is cut into
-// G groups of L lanes, each lane owning a 16-byte slice of a rank-R row, and
-// the block into G equal contiguous runs, one per group.  Each group streams
-// its run through the warp's shared-memory ring: its leader lane issues 1D
-// bulk-async copies (cp.async.bulk) of the next K nonzeros and of their remap
-// ids S-1 tiles ahead, completion is counted on per-warp mbarriers (one
-// arrival per group), and every wait is bounded.  For every tile:
-//   * remap (Algorithm 3): the group's lanes copy its nonzeros to their places
-//     in the next mode's order, T_out[next_pos[p]] = x_p;
-//   * elementwise computation (Algorithm 2): the group walks its segment U
-//     nonzeros at a time, issues all gathers A_k[i_k, slice] (k != n, 16-byte
-//     read-only loads; indices come from shared memory) into packed
-//     registers, then accumulates val * Hadamard product in order while the
-//     output row is unchanged; rows that start and end inside the run are
-//     written straight to M_n, and the run state carries over to the next
-//     tile.
-// At the end of the block the first and last row of every run, left as
-// partial sums in shared memory, are added by the warp in run order; a row
-// that continues past the block is written as a partial to `part` and summed
-// by the fix-up kernel in block order.  No atomics: results are bit-identical
-// from run to run and every output row is written exactly once (empty rows are
-// zero-filled by the writer of the next nonempty row, or of the last one).
+// A block [lo, hi) of the mode-n ordered working copy (the paper's thread block over a
+// tensor partition, Algorithm 4, shrunk so far that no CTA-wide synchronisation is
+// needed) is one warp's work.  The resident warps take the blocks in order: two each to
+// begin with, then whatever a counter hands out, claimed a block ahead.  Lane 0 streams
+// the warp's blocks tile by tile through a shared-memory ring by 1D bulk-async copies
+// (cp.async.bulk) of the nonzeros and of their remap ids, completion is counted on
+// per-warp mbarriers, and every wait is bounded.
+//   * Remap (Algorithm 3): when a tile has landed, the warp's lanes copy its nonzeros
+//     to their places in the next mode's order, T_out[next_pos[p]] = x_p.  Because the
+//     blocks are small and taken in order, the warps store near each other's places in
+//     the next order at nearly the same time, and L2 gathers sectors into whole lines
+//     before it writes them (a lone 32-byte sector costs DRAM as much as its line).
+//   * Elementwise computation (Algorithm 2): the warp is cut into G groups of L lanes,
+//     each lane owning a slice of a rank-R row.  Nonzero u G + g of a chunk of U G
+//     consecutive ones is step u of group g.  The ring holds the gathered slices
+//     A_k[i_k, slice] (k != n) of one chunk: as each step is consumed, its place takes
+//     the gathers of the same step of the next chunk, across tile and block ends, so
+//     the warp always has close to U G nonzeros' rows in flight and never drains.
+//     Neighbouring nonzeros of one row often share a fiber index, and the groups then
+//     gather the same line in one request.
+//   * Rows: while the output row does not change, the groups add to G partial rows in
+//     registers, which are added when the row ends.  Chunks in which it changes put
+//     their weighted products in a shared-memory scratch, and a short loop adds them
+//     row by row.  The block's first and last row, where they continue outside the
+//     block, are left as partials in `part`, summed by the fix-up kernel in block order.
+// No atomics on data (the counter only hands out blocks, and a block's result does not
+// depend on who takes it): results are bit-identical from run to run and every output
+// row is written exactly once (empty rows are zero-filled by the writer of the next
+// nonempty row, or of the last one).
+//
+// What bounds it, measured on a GB300 (3 modes 120000 x 90000 x 2000000, 100M nonzeros,
+// Zipf 1.1, rank 32 FP32; ms per pass of mode 0 / 1 / 2): 2.55 / 2.89 / 2.46 with the
+// remap and 1.43 / 1.43 / 1.81 without, against 2.98 / 3.26 / 2.58 and 1.91 / 1.95 /
+// 1.72 of one 1.7K-nonzero block per warp with its groups on four separate runs.  Three
+// things set the shape:
+//   * Shared memory is taken from L1, and the gathers in flight (up to 128 KB per SM)
+//     need L1 lines to land in: a 128-nonzero tile and a 4 KB scratch per warp left
+//     modes 0 and 1 at 2.1-2.2 ms without the remap, 64 and 2 KB take 1.4.
+//   * Blocks of about 512 nonzeros: larger ones spread the remap stores over more of
+//     the next order than L2 holds, smaller ones pay more for their ends.
+//   * Code size: with the row ends' code unrolled into every step the kernel was 50-66
+//     KB, and mode 2 (50 nonzeros per row) waited on instruction fetch at 2.9 ms; as a
+//     loop over the scratch it is 36 KB.
+// The remainder is gather latency and the DRAM cost of the scattered sectors.
 #pragma once
 
 #include "mttkrp_common.cuh"
@@ -35,132 +55,47 @@ namespace spm {
 constexpr int kMaxStages = 4;  // tiles per warp ring: stages - 1 in flight while one is used
 constexpr int kWarps = kThreads / 32;
 
-// Per-warp shared-memory layout (bytes, in order).
+// Per-warp shared-memory layout (bytes, in order): the staged tiles, their remap
+// ids, the row scratch, one descriptor per stage, and the mbarriers.
 struct WarpLayout {
-  size_t ebuf, npbuf, sacc, cacc, srow, sprev, mbar, total;
+  size_t ebuf, npbuf, scratch, rows, desc, mbar, total;
 };
 
-// Remap ids staged per group segment of k nonzeros: k + 3 ids at most (the
-// copy starts at the 16-byte boundary at or below the segment) rounded up to a
-// multiple of 4 ints, so that every bulk-copy destination stays 16-byte aligned.
+// Row scratch of a warp: the weighted products of HS steps' nonzeros (floats; 2 KB, see
+// above), and the places in them where rows begin.
+constexpr int kScratch = 512;
+__host__ __device__ constexpr int scratch_steps(int NV, int U) {
+  return kScratch / (32 * NV) < U ? kScratch / (32 * NV) : U;
+}
+
+// Remap ids staged per tile of k nonzeros: k + 3 ids at most (the copy starts at
+// the 16-byte boundary at or below the tile) rounded up to a multiple of 4 ints, so
+// that every bulk-copy destination stays 16-byte aligned.
 __host__ __device__ inline int np_stage_ints(int tw) { return (tw + 8 + 3) & ~3; }
 
-__host__ __device__ inline WarpLayout warp_layout(int es, int tw, int R, int G, int stages) {
+__host__ __device__ inline WarpLayout warp_layout(int es, int tw, int stages, bool ids) {
   WarpLayout l;
   size_t o = 0;
   l.ebuf = o;
   o += (size_t)stages * tw * es;
   l.npbuf = o;
-  o += (size_t)stages * G * np_stage_ints(tw / G) * 4;
-  l.sacc = o;
-  o += (size_t)2 * G * R * 4;
-  l.cacc = o;
-  o += (size_t)R * 4;
-  l.srow = o;
-  o += (size_t)2 * G * 4;
-  l.sprev = o;
-  o += (size_t)2 * G * 4;
-  o = (o + 7) & ~(size_t)7;
+  if (ids) o += (size_t)stages * np_stage_ints(tw) * 4;
+  l.scratch = o;
+  o += (size_t)kScratch * 4;
+  l.rows = o;
+  o += (size_t)36 * 4;
+  l.desc = o;
+  o += (size_t)stages * 16;
   l.mbar = o;
   o += (size_t)(stages + 1) * 8;  // the ring, plus one barrier only the stall test waits on
   l.total = (o + 127) & ~(size_t)127;
   return l;
 }
 
-
-// Registers a gathered factor-row slice lands in before it is used: one
-// 16-byte vector (4 FP32 or 8 packed BF16) on the vector path, RC scalars on
-// the scalar path.  Keeping BF16 packed until use halves the registers that
-// loads in flight occupy.
-template <typename T, int VW, int RC>
-struct Landing {
-  using type = uint4;
-  __device__ __forceinline__ static void load(const void* base, int64_t row, int R, int sub,
-                                              int L, uint64_t pol, type& out) {
-    if (sub * VW < R)
-      out = ld_nc_hint_v4(reinterpret_cast<const uint4*>(static_cast<const T*>(base) + row * R) +
-                              sub,
-                          pol);
-    else
-      out = make_uint4(0u, 0u, 0u, 0u);
-  }
-  __device__ __forceinline__ static void unpack(const type& v, float* x) {
-    if constexpr (VW == 4) {
-      x[0] = __uint_as_float(v.x);
-      x[1] = __uint_as_float(v.y);
-      x[2] = __uint_as_float(v.z);
-      x[3] = __uint_as_float(v.w);
-    } else {
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        x[2 * j] = __uint_as_float(w[j] << 16);
-        x[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
-      }
-    }
-  }
-};
-
-// BF16 rows in 8-byte lane slices (4 values per lane)
-template <>
-struct Landing<__nv_bfloat16, 4, 1> {
-  using type = uint2;
-  __device__ __forceinline__ static void load(const void* base, int64_t row, int R, int sub,
-                                              int L, uint64_t pol, type& out) {
-    if (sub * 4 < R)
-      out = ld_nc_hint_v2(
-          reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(base) + row * R) + sub,
-          pol);
-    else
-      out = make_uint2(0u, 0u);
-  }
-  __device__ __forceinline__ static void unpack(const type& v, float* x) {
-    x[0] = __uint_as_float(v.x << 16);
-    x[1] = __uint_as_float(v.x & 0xffff0000u);
-    x[2] = __uint_as_float(v.y << 16);
-    x[3] = __uint_as_float(v.y & 0xffff0000u);
-  }
-};
-
-// One lane's slice of a factor row at ptr (16 or 8 bytes); with `flagged`, the L1
-// choice of a hot-row flag (keep: evict_last; else evict_first).
-template <typename LT>
-__device__ __forceinline__ LT load_lane(const uint8_t* ptr, uint64_t pol, bool flagged, bool keep);
-template <>
-__device__ __forceinline__ uint4 load_lane<uint4>(const uint8_t* ptr, uint64_t pol, bool flagged,
-                                                  bool keep) {
-  return flagged ? ld_nc_l1_v4(ptr, pol, keep) : ld_nc_hint_v4(ptr, pol);
-}
-template <>
-__device__ __forceinline__ uint2 load_lane<uint2>(const uint8_t* ptr, uint64_t pol, bool flagged,
-                                                  bool keep) {
-  return flagged ? ld_nc_l1_v2(ptr, pol, keep) : ld_nc_hint_v2(ptr, pol);
-}
-
-template <typename T, int RC>
-struct Landing<T, 1, RC> {
-  struct type {
-    float v[RC];
-  };
-  __device__ __forceinline__ static void load(const void* base, int64_t row, int R, int sub,
-                                              int L, uint64_t, type& out) {
-#pragma unroll
-    for (int j = 0; j < RC; ++j) {
-      const int r = sub + L * j;
-      out.v[j] = r < R ? load_scalar<T>(base, row * R + r) : 0.f;
-    }
-  }
-  __device__ __forceinline__ static void unpack(const type& v, float* x) {
-#pragma unroll
-    for (int j = 0; j < RC; ++j) x[j] = v.v[j];
-  }
-};
-
-// NT: modes at compile time (0 = runtime); T: factor type; VW: values per lane
-// per 16-byte load (1 = scalar path); RC: rank chunks per lane (scalar path);
-// U: nonzeros in flight per lane group; MODE: output mode at compile time (3
-// modes only; -1 = runtime); ESB: element bytes when fixed (0 = the smallest
-// multiple of 16 that holds N indices and the value).
+// NT: modes at compile time (0 = runtime); T: factor type; VW, RC: values per piece and
+// pieces of a row per lane (Piece); U: steps in flight; MODE: output mode at compile
+// time (3 modes only; -1 = runtime); ESB: element bytes when fixed (0: 32, or 16 for
+// packed nonzeros (PK), with 4 to 6 modes at compile time; else the plan's).
 // LOSS (3 modes, 16- or 32-byte nonzeros): the fused first pass of the CP loss.  Each
 // nonzero's own factor row A_n[i_n] is gathered as well; the model value
 // m_e = sum_r prod_k A_k[i_k, r] and the residual e = m_e - x_e replace the
@@ -289,669 +224,802 @@ __device__ __forceinline__ void remap_warp_tiles(const MttkrpArgs& a, int mode, 
   }
 }
 
-// A lane group's change of output row on the vector path (VW values a lane, VW
-// >= 4): the row that ends (cur, partial sums acc) goes to the group's head slot
-// if it is the run's first row, else straight to M_n after the empty rows before
-// it (and, for the mode's last row, the empty rows after it).  Returns the run's
-// previous row and head flag.  Kept out of line: the batch code, unrolled over its
-// nonzeros, carries one call per nonzero instead of a copy of this.
-template <int VW>
-struct RowAcc {
-  float v[VW];
-};
-template <int VW>
-__device__ __noinline__ int2 close_row(RowAcc<VW> acc, int cur, int prev_in_run, int head,
-                                       float* __restrict__ out, int R, int sub, float sc,
-                                       int last_row, int64_t out_rows, int no_fill, int slot,
-                                       int* __restrict__ srow, int* __restrict__ sprev,
-                                       float* __restrict__ sacc) {
-  const bool live = sub * VW < R;
-  if (head) {
-    if (cur >= 0) {
-      if (sub == 0) {
-        srow[slot] = cur;
-        sprev[slot] = -2;
-      }
-#pragma unroll
-      for (int j = 0; j < VW; ++j)
-        if (sub * VW + j < R) sacc[(size_t)slot * R + sub * VW + j] = acc.v[j];
-      head = 0;
-    }
-  } else {
-    if (!no_fill && live)
-      for (int64_t z = (int64_t)prev_in_run + 1; z < cur; ++z) {
-        float4* d = reinterpret_cast<float4*>(out + z * R + sub * VW);
-#pragma unroll
-        for (int q = 0; q < VW / 4; ++q) d[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    if (live) {
-      float4* d = reinterpret_cast<float4*>(out + (int64_t)cur * R + sub * VW);
-#pragma unroll
-      for (int q = 0; q < VW / 4; ++q)
-        d[q] = make_float4(acc.v[4 * q] * sc, acc.v[4 * q + 1] * sc, acc.v[4 * q + 2] * sc,
-                           acc.v[4 * q + 3] * sc);
-    }
-    if (cur == last_row && !no_fill && live)
-      for (int64_t z = (int64_t)cur + 1; z < out_rows; ++z) {
-        float4* d = reinterpret_cast<float4*>(out + z * R + sub * VW);
-#pragma unroll
-        for (int q = 0; q < VW / 4; ++q) d[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+// A lane's share of a factor row: RC pieces of VW consecutive values, piece j
+// starting at value (sub + L j) VW.  One load per piece: 16 bytes (4 FP32 or 8
+// BF16), 8 bytes (2 or 4) or a 4- or 2-byte load where the rank or the factors'
+// alignment allows no more.  BF16 stays packed until use.
+template <typename T, int VW>
+struct Piece;
+template <>
+struct Piece<float, 4> {
+  using type = uint4;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t pol) {
+    return ld_nc_hint_v4(p, pol);
   }
-  if (cur >= 0) prev_in_run = cur;
-  return make_int2(prev_in_run, head);
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    x[0] = __uint_as_float(v.x);
+    x[1] = __uint_as_float(v.y);
+    x[2] = __uint_as_float(v.z);
+    x[3] = __uint_as_float(v.w);
+  }
+};
+template <>
+struct Piece<float, 2> {
+  using type = uint2;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t pol) {
+    return ld_nc_hint_v2(p, pol);
+  }
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    x[0] = __uint_as_float(v.x);
+    x[1] = __uint_as_float(v.y);
+  }
+};
+template <>
+struct Piece<float, 1> {
+  using type = uint32_t;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t pol) {
+    return ld_nc_hint_v1(p, pol);
+  }
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    x[0] = __uint_as_float(v);
+  }
+};
+template <>
+struct Piece<__nv_bfloat16, 2> {
+  using type = uint32_t;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t pol) {
+    return ld_nc_hint_v1(p, pol);
+  }
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    x[0] = __uint_as_float(v << 16);
+    x[1] = __uint_as_float(v & 0xffff0000u);
+  }
+};
+template <>
+struct Piece<__nv_bfloat16, 4> {
+  using type = uint2;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t pol) {
+    return ld_nc_hint_v2(p, pol);
+  }
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    Piece<__nv_bfloat16, 2>::unpack(v.x, x);
+    Piece<__nv_bfloat16, 2>::unpack(v.y, x + 2);
+  }
+};
+template <>
+struct Piece<__nv_bfloat16, 8> {
+  using type = uint4;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t pol) {
+    return ld_nc_hint_v4(p, pol);
+  }
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    Piece<__nv_bfloat16, 2>::unpack(v.x, x);
+    Piece<__nv_bfloat16, 2>::unpack(v.y, x + 2);
+    Piece<__nv_bfloat16, 2>::unpack(v.z, x + 4);
+    Piece<__nv_bfloat16, 2>::unpack(v.w, x + 6);
+  }
+};
+template <>
+struct Piece<__nv_bfloat16, 1> {
+  using type = uint32_t;
+  __device__ __forceinline__ static type load(const uint8_t* p, uint64_t) {
+    return (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p));
+  }
+  __device__ __forceinline__ static void unpack(const type& v, float* x) {
+    x[0] = __uint_as_float(v << 16);
+  }
+};
+
+// Stores the VW consecutive values of one piece, times sc.
+template <int VW>
+__device__ __forceinline__ void store_piece(float* __restrict__ d, const float* v, float sc) {
+  if constexpr (VW % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < VW / 4; ++q)
+      reinterpret_cast<float4*>(d)[q] = make_float4(v[4 * q] * sc, v[4 * q + 1] * sc,
+                                                    v[4 * q + 2] * sc, v[4 * q + 3] * sc);
+  } else if constexpr (VW == 2) {
+    *reinterpret_cast<float2*>(d) = make_float2(v[0] * sc, v[1] * sc);
+  } else {
+    d[0] = v[0] * sc;
+  }
+}
+
+// CTAs per SM the register budget is cut for.  Wide lanes (16 bytes of every
+// gathered row in flight) take 128 registers and two CTAs; lanes that hold at most 24
+// registers in flight take three.
+template <int NT, int VW, int RC, int U, bool LOSS>
+constexpr int warp_min_ctas() {
+  return NT > 0 && VW * RC <= 2 && U * (NT - 1) * VW * RC <= 24 ? 3 : 2;
 }
 
 template <int NT, typename T, int VW, int RC, int U, int MODE, int ESB = 0, bool LOSS = false,
-          bool RWARP = false>
-__global__ void __launch_bounds__(kThreads, ((U <= 4 && VW > 1 && NT <= 3 && !LOSS) ? 3 : 2))
+          bool RWARP = false, bool PK = false>
+__global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>()))
     mttkrp_warp_kernel(const MttkrpArgs a, const int L) {
-  static_assert(!LOSS || (NT == 3 && MODE >= 0 && VW > 1 && (ESB == 32 || ESB == 16)),
+  static_assert(!LOSS || (NT == 3 && MODE >= 0 && VW > 1 && U == 4 && (ESB == 32 || ESB == 16)),
                 "the fused CP-loss pass is built for 3 modes and 16- or 32-byte nonzeros");
   static_assert(!RWARP || (NT == 3 && MODE >= 0 && VW > 1 && ESB == 32 && !LOSS),
                 "the remap warp is built for 3 modes and 32-byte nonzeros");
+  static_assert(!PK || NT >= 4, "packed nonzeros have 4 or more modes");
   constexpr int CW = RWARP ? kWarps - 1 : kWarps;  // warps that compute
   constexpr int NV = VW * RC;
   const int N = NT > 0 ? NT : a.nmodes;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int G = 32 / L, sub = lane % L, gw = lane / L;
-  // element stride: a compile-time constant when the number of modes is
-  // (packed nonzeros of 4 or more modes are 16 bytes: the plan's stride)
-  constexpr int ES_C = ESB > 0 ? ESB : (NT > 0 ? (((4 * NT + 4) + 15) & ~15) : 0);
-  const int es = (NT > 0 && !a.pk.packed) ? ES_C : a.es;
+  // element stride: a compile-time constant when the layout is
+  constexpr int ES_C = ESB > 0 ? ESB : (NT >= 4 ? (PK ? 16 : 32) : 0);
+  const int es = ES_C > 0 ? ES_C : a.es;
   const int R = a.R, mode = MODE >= 0 ? MODE : a.mode;
-  const int TW = a.tile, K = TW / G, NPK = np_stage_ints(K);
+  const int TW = a.tile, NPK = np_stage_ints(TW);
+  const bool remap = a.elems_out != nullptr && !RWARP;  // RWARP: the remap warp's work
+  const bool ids = remap && !a.alpha_word;              // remap ids from the next_pos array
+  const int S = a.stages;
+  const WarpLayout lay = warp_layout(es, TW, S, a.alpha_word == 0);
   if constexpr (RWARP) {
     if (warp == kWarps - 1) {
       extern __shared__ __align__(128) uint8_t smem_r[];
-      const WarpLayout lr = warp_layout(es, TW, R, G, a.stages);
       if (a.elems_out)
-        remap_warp_tiles(a, MODE, CW, smem_r + (size_t)CW * lr.total,
+        remap_warp_tiles(a, MODE, CW, smem_r + (size_t)CW * lay.total,
                          a.wait_ns ? a.wait_ns : kWaitLimitNs);
       return;
     }
   }
-  const int wb = blockIdx.x * CW + warp;
-  if (wb >= a.nblk) return;
-  const int4 bi = a.blkinfo[wb];
-  const int lo = bi.x, hi = bi.y;
-  if (lo >= hi) {
-    if (LOSS && lane == 0) a.loss_part[wb] = 0.0;
-    return;
-  }
+  const int nwarps = gridDim.x * CW;  // blocks w, w + nwarps, ... belong to warp w
 
   extern __shared__ __align__(128) uint8_t smem[];
-  const int S = a.stages;
-  const WarpLayout lay = warp_layout(es, TW, R, G, S);
   uint8_t* wbase = smem + (size_t)warp * lay.total;
   uint8_t* ebuf = wbase + lay.ebuf;
   int32_t* npbuf = reinterpret_cast<int32_t*>(wbase + lay.npbuf);
-  float* sacc = reinterpret_cast<float*>(wbase + lay.sacc);
-  float* cacc = reinterpret_cast<float*>(wbase + lay.cacc);  // carry row partial (lanes over R)
-  int* srow = reinterpret_cast<int*>(wbase + lay.srow);
-  int* sprev = reinterpret_cast<int*>(wbase + lay.sprev);
+  float* scratch = reinterpret_cast<float*>(wbase + lay.scratch);
+  int* srows = reinterpret_cast<int*>(wbase + lay.rows);
+  int4* desc = reinterpret_cast<int4*>(wbase + lay.desc);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(wbase + lay.mbar);
 
-  // this group's run [ga, gb) of the block
-  const int64_t len = hi - lo;
-  const int ga = lo + (int)(len * gw / G), gb = lo + (int)(len * (gw + 1) / G);
-  const int maxrun = (int)((len + G - 1) / G);
-  const int ntiles = (maxrun + K - 1) / K;
-  const bool remap = a.elems_out != nullptr && !RWARP;  // RWARP: the remap warp's work
-  const bool leader = (sub == 0);
   const float sc = a.scale ? __ldg(a.scale) : 1.0f;
-  const int64_t out_rows = a.out_rows;
   float* __restrict__ out = a.out;
   // L2 policies: the element stream, remap ids and remapped copy are touched
   // once per mode (evict first); factor rows are reused (evict last)
   const uint64_t pol_stream = make_policy((a.hints & 1) ? 1 : 0);
   const uint64_t pol_factor = make_policy((a.hints & 2) ? 2 : 0);
-  // static 3-mode vector path: this lane's slice (VW values) of the two input
-  // factors' rows (lanes past R read slice 0; their values are never stored)
   const uint32_t rowb = (uint32_t)R * (uint32_t)sizeof(T);
-  constexpr int LB = VW * (int)sizeof(T);  // bytes of a lane's slice (16, or 8 for BF16 VW 4)
-  const uint8_t* lane_base[2];
-  {
-    const int lsub = (sub * VW < R) ? sub : 0;
-    const int k1 = (MODE >= 0 ? MODE : 0) + 1, k2 = (MODE >= 0 ? MODE : 0) + 2;
-    lane_base[0] = static_cast<const uint8_t*>(a.factors[k1 % 3 < N ? k1 % 3 : 0]) + lsub * LB;
-    lane_base[1] = static_cast<const uint8_t*>(a.factors[k2 % 3 < N ? k2 % 3 : 0]) + lsub * LB;
-  }
-  // fused CP loss: this lane's slice of the output mode's own factor, and the
-  // lane's running sum of squared residuals (FP32 per batch, FP64 across)
-  const uint8_t* own_base = nullptr;
-  const bool lane_live = sub * VW < R;
-  double lsum = 0.0;
-  if constexpr (LOSS)
-    own_base = static_cast<const uint8_t*>(a.factors[MODE]) + (lane_live ? sub : 0) * LB;
-
-  // the group's leader stages the group's segment of tile t (one mbarrier
-  // arrival per group and tile, with the segment's byte count)
-  auto issue = [&](int t) {
-    const int st = t % S;
-    const int seg = ga + t * K;
-    const int n = max(0, min(K, gb - seg));
-    uint32_t ebytes = (uint32_t)n * es, npbytes = 0;
-    int np0 = 0;
-    if (remap && !a.alpha_word && n > 0) {  // remap ids from the next_pos array
-      np0 = seg & ~3;
-      npbytes = ((uint32_t)(seg + n - np0) * 4u + 15u) & ~15u;
-    }
-    fence_proxy_async_smem();
-    mbar_expect_tx(&mbar[st], ebytes + npbytes);
-    if (n > 0) {
-      bulk_g2s_hint(ebuf + ((size_t)st * TW + (size_t)gw * K) * es, a.elems_in + (size_t)seg * es,
-                    ebytes, &mbar[st], pol_stream);
-      if (npbytes)
-        bulk_g2s_hint(npbuf + (st * G + gw) * NPK, a.next_pos + np0, npbytes, &mbar[st],
-                      pol_stream);
-    }
-  };
-
-  if (lane == 0) {
-    for (int b = 0; b <= S; ++b) mbar_init(&mbar[b], G);  // mbar[S]: never completed
-    fence_mbar_init();
-  }
-  __syncwarp();
-  if (leader)
-    for (int q = 0; q < S - 1 && q < ntiles; ++q) issue(q);
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
 
-  auto rank_of = [&](int j) -> int {
-    if constexpr (VW > 1) return sub * VW + j;
-    return sub + L * j;
+  // ---- staging.  Lane 0 walks the warp's blocks tile by tile, one stage each: a
+  // descriptor {first position, nonzeros | flags << 16, block, row before the
+  // block}, then one mbarrier arrival with the tile's byte count.  A tile of no
+  // nonzeros ends the sequence.
+  constexpr int kFirst = 4, kLast = 8;  // tile flags beside BLK_HEAD_SPLIT, BLK_TAIL_SPLIT
+  int in_flight = 0;                    // tiles issued and not yet waited for
+  // lane 0: block and position, the next block and its descriptor, the one after
+  int ib = 0, ipos = 0, ihi = 0, ib1 = blockIdx.x * CW + warp, ib2 = ib1 + nwarps;
+  int4 ibi = make_int4(0, 0, 0, 0), inext = make_int4(0, 0, 0, 0);
+  if (lane == 0) {
+    for (int q = 0; q <= S; ++q) mbar_init(&mbar[q], 1);  // mbar[S]: never completed
+    fence_mbar_init();
+    if (ib1 < a.nblk) inext = a.blkinfo[ib1];
+  }
+  __syncwarp();
+  auto issue = [&](int st) {  // into stage st
+    if (lane == 0) {
+      while (ipos >= ihi && ib1 < a.nblk) {  // the next block that holds nonzeros
+        ib = ib1;
+        ibi = inext;
+        ipos = ibi.x;
+        ihi = ibi.y;
+        ib1 = ib2;  // both are used one block later
+        if (ib1 < a.nblk) inext = a.blkinfo[ib1];
+        if (ib1 < a.nblk && a.nblk > 2 * nwarps) ib2 = 2 * nwarps + atomicAdd(a.sched, 1);
+        else ib2 = a.nblk;
+        if (LOSS && ipos >= ihi) a.loss_part[ib] = 0.0;
+      }
+      const int n = ipos < ihi ? min(TW, ihi - ipos) : 0;
+      const int fl = ibi.w | (ipos == ibi.x ? kFirst : 0) | (ipos + n == ihi ? kLast : 0);
+      desc[st] = make_int4(ipos, n | (fl << 16), ib, ibi.z);
+      const uint32_t ebytes = (uint32_t)n * es;
+      uint32_t npbytes = 0;
+      const int np0 = ipos & ~3;
+      if (ids && n > 0) npbytes = ((uint32_t)(ipos + n - np0) * 4u + 15u) & ~15u;
+      fence_proxy_async_smem();
+      mbar_expect_tx(&mbar[st], ebytes + npbytes);
+      if (n > 0) {
+        bulk_g2s_hint(ebuf + (size_t)st * TW * es, a.elems_in + (size_t)ipos * es, ebytes,
+                      &mbar[st], pol_stream);
+        if (npbytes)
+          bulk_g2s_hint(npbuf + st * NPK, a.next_pos + np0, npbytes, &mbar[st], pol_stream);
+      }
+      ipos += n;
+    }
+    ++in_flight;
   };
-  auto zero_rows_group = [&](int64_t from, int64_t to) {
-    if (a.no_fill) return;  // Algorithm 1 blocks: empty rows are zeroed from a list
-    for (int64_t z = from; z < to; ++z) {
-      if constexpr (VW > 1) {
-        if (sub * VW < R) {
-          float4* d = reinterpret_cast<float4*>(out + z * R + sub * VW);
-#pragma unroll
-          for (int q = 0; q < VW / 4; ++q) d[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-          const int r = rank_of(j);
-          if (r < R) out[z * R + r] = 0.f;
+  for (int st = 0; st < S; ++st) issue(st);
+
+  // Waits for the oldest tile not yet waited for, in stage st with mbarrier phase
+  // `phase`; false (after recording the error and awaiting, bounded, the
+  // copies still in flight) when its copy did not complete in time.
+  bool stall = a.stall_test;  // waits first on mbar[S], which no copy and no thread completes
+  auto wait_tile = [&](int st, uint32_t phase) -> bool {
+    const bool ok = mbar_wait_bounded(&mbar[stall ? S : st], stall ? 0u : phase, wait_ns);
+    stall = false;
+    if (__all_sync(0xffffffffu, ok)) {
+      --in_flight;
+      return true;
+    }
+    if (lane == 0) {
+      atomicOr(a.err, 1);
+      for (; in_flight > 0; --in_flight) {
+        (void)mbar_wait_bounded(&mbar[st], phase);
+        if (++st == S) {
+          st = 0;
+          phase ^= 1u;
         }
       }
     }
+    return false;
   };
-  auto write_row_group = [&](int row, const float* acc, int prev) {
-    zero_rows_group((int64_t)prev + 1, row);
-    if constexpr (VW > 1) {
-      if (sub * VW < R) {
-        float4* d = reinterpret_cast<float4*>(out + (int64_t)row * R + sub * VW);
-#pragma unroll
-        for (int q = 0; q < VW / 4; ++q)
-          d[q] = make_float4(acc[4 * q] * sc, acc[4 * q + 1] * sc, acc[4 * q + 2] * sc,
-                             acc[4 * q + 3] * sc);
+
+  auto do_remap = [&](int st) {  // Algorithm 3: a tile's nonzeros to their places in the next order
+    const int4 d = desc[st];
+    const int n = d.y & 0xffff;
+    const uint8_t* eb = ebuf + (size_t)st * TW * es;
+    const int32_t* np = npbuf + st * NPK + (d.x & 3);
+    if (es % 32 == 0) {  // whole 32-byte sectors per store (no read of the old sector)
+      const int nv = es >= 32 ? es / 32 : 1;
+      const int aw = a.alpha_word;  // remap id carried in the staged nonzero (Section 3.5)
+      for (int i = lane; i < n * nv; i += 32) {
+        const int e = (nv == 1) ? i : i / nv, c = (nv == 1) ? 0 : i - e * nv;
+        const uint4* src = reinterpret_cast<const uint4*>(eb + (size_t)e * es) + 2 * c;
+        const uint4 lo4 = src[0], hi4 = src[1];
+        // with the ids in the nonzero (32-byte stride, one sector: c == 0) the id is
+        // word aw of the sector, i.e. component aw - 4 of its upper half
+        // (bit 31 of the id words is a hot-row flag, not part of the id)
+        const int dst = aw ? (int)((aw == 4 ? hi4.x : (aw == 5 ? hi4.y : hi4.z)) & 0x7fffffffu)
+                           : np[e];
+        st_hint_v8(a.elems_out + (size_t)dst * es + 32 * c, lo4, hi4, pol_stream);
       }
     } else {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        const int r = rank_of(j);
-        if (r < R) out[(int64_t)row * R + r] = acc[j] * sc;
+      const int nv = es / 16;  // 16-byte vectors per element
+      for (int i = lane; i < n * nv; i += 32) {
+        const int e = (nv == 1) ? i : i / nv, c = (nv == 1) ? 0 : i - e * nv;
+        const uint4 v = reinterpret_cast<const uint4*>(eb + (size_t)e * es)[c];
+        st_hint_v4(reinterpret_cast<uint4*>(a.elems_out + (size_t)np[e] * es) + c, v, pol_stream);
       }
-    }
-    if (row == a.last_row) zero_rows_group((int64_t)row + 1, out_rows);
-  };
-  auto store_slot = [&](int s, int row, int prev, const float* acc) {
-    if (sub == 0) {
-      srow[s] = row;
-      sprev[s] = prev;
-    }
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      const int r = rank_of(j);
-      if (r < R) sacc[(size_t)s * R + r] = acc[j];
     }
   };
 
-  // run state of this group, carried from tile to tile
+  // fields of the staged nonzero at ep
+  uint32_t foff[NT > 0 ? NT : 1];  // plain nonzeros: byte offsets of the fields (output row first)
+#pragma unroll
+  for (int j = 0; j < (NT > 0 ? NT : 1); ++j) {
+    int k = mode + j;
+    if (k >= N) k -= N;
+    foff[j] = 4u * (uint32_t)k;
+  }
+  auto row_of = [&](const uint8_t* ep) -> int {
+    if constexpr (PK || NT == 0) {
+      return elem_index(ep, mode, a.pk);
+    } else if constexpr (MODE >= 0) {
+      return reinterpret_cast<const int*>(ep)[MODE];
+    } else {
+      return *reinterpret_cast<const int*>(ep + foff[0]);
+    }
+  };
+  // ---- output rows.  The warp's current row `cur` is summed in G parts (acc of each
+  // lane group), which are added when the row ends.  Steps in which rows change put
+  // their weighted products into the scratch; every HS steps these are added to their
+  // rows in a loop (unrolled with the steps, the row ends' code outgrew the instruction
+  // cache).
+  constexpr int HS = scratch_steps(NV, U);
+  static_assert(HS >= 1 && U % HS == 0, "the scratch holds whole steps");
   float acc[NV];
 #pragma unroll
   for (int j = 0; j < NV; ++j) acc[j] = 0.f;
-  int cur = -1;
-  bool head = true;
-  int prev_in_run = -1;
-  const uint8_t* eb = nullptr;  // this group's segment of the current tile
-
-  constexpr int NI = (NT > 0 ? NT : 2) - 1;
-  auto batch = [&](int e, int nb) {
-    // 1) element fields from shared memory, 2) every gather of the batch
-    // issued into packed registers, 3) products consumed in order
-    int rows[U];
-    float vals[U];
-    int ixs[U][NI];
+  int cur = -1, prev = -1;  // current row, the nonempty row before it
+  bool first = true;        // cur is the block's first row
+  auto piece_rank = [&](int j) -> int { return (sub + L * j) * VW; };  // first value of piece j
+  auto store_row = [&](float* d, const float (&v)[NV], float s) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (u < nb) {
-        const uint8_t* ep = eb + (size_t)(e + u) * es;
-        if constexpr (NT == 3 && MODE >= 0) {
-          const int4 v = *reinterpret_cast<const int4*>(ep);
-          const int f[3] = {v.x, v.y, v.z};
-          rows[u] = f[MODE];
-          ixs[u][0] = f[(MODE + 1) % 3];
-          ixs[u][1] = f[(MODE + 2) % 3];
-          vals[u] = __int_as_float(v.w);
-        } else if (a.pk.packed) {  // 4-6 modes in 16 bytes (bit fields)
-          const uint4 w4 = *reinterpret_cast<const uint4*>(ep);
-          const uint32_t w[3] = {w4.x, w4.y, w4.z};
-          rows[u] = (int)pk_field(w, a.pk.off[mode], a.pk.bits[mode]);
-          vals[u] = __uint_as_float(w4.w);
-          int k = mode;
+    for (int j = 0; j < RC; ++j)
+      if (piece_rank(j) < R) store_piece<VW>(d + piece_rank(j), v + j * VW, s);
+  };
+  auto add_slot = [&](int k, float (&v)[NV]) {  // v += this lane's pieces of scratch row k
 #pragma unroll
-          for (int j = 0; j < NI; ++j) {
-            if (j < N - 1) {
-              k = (k + 1 == N) ? 0 : k + 1;
-              ixs[u][j] = (int)pk_field(w, a.pk.off[k], a.pk.bits[k]);
-            }
-          }
-        } else {
-          const int* el = reinterpret_cast<const int*>(ep);
-          rows[u] = el[mode];
-          vals[u] = __int_as_float(el[N]);
-          int k = mode;
+    for (int j = 0; j < RC; ++j) {
+      const int c = piece_rank(j) < R ? piece_rank(j) : 0;
+      const float* x = scratch + k * R + c;
+      if constexpr (VW % 4 == 0) {
 #pragma unroll
-          for (int j = 0; j < NI; ++j) {
-            if (j < N - 1) {
-              k = (k + 1 == N) ? 0 : k + 1;
-              ixs[u][j] = el[k];
-            }
-          }
+        for (int q = 0; q < VW / 4; ++q) {
+          const float4 t = reinterpret_cast<const float4*>(x)[q];
+          v[j * VW + 4 * q] += t.x;
+          v[j * VW + 4 * q + 1] += t.y;
+          v[j * VW + 4 * q + 2] += t.z;
+          v[j * VW + 4 * q + 3] += t.w;
         }
+      } else {
+#pragma unroll
+        for (int q = 0; q < VW; ++q) v[j * VW + q] += x[q];
       }
     }
-    typename Landing<T, VW, RC>::type raw[U][NI];
-    typename Landing<T, VW, RC>::type rown[LOSS ? U : 1];  // A_n[i_n] slices (fused loss)
-    float hh[LOSS ? U : 1][NV];  // fused loss: the product of the two gathered slices
-    if constexpr (LOSS) {
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (u < nb)
-          rown[u] = load_lane<typename Landing<T, VW, RC>::type>(
-              own_base + (uint64_t)(uint32_t)rows[u] * rowb, pol_factor, false, false);
-    }
-    if constexpr (NT == 3 && MODE >= 0 && VW > 1) {
-      // static modes: one 32 x 32 -> 64-bit multiply per row address
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (u < nb) {
-            using LT = typename Landing<T, VW, RC>::type;
-            raw[u][j] = load_lane<LT>(lane_base[j] + (uint64_t)(uint32_t)ixs[u][j] * rowb,
-                                      pol_factor, false, false);
-          }
+  };
+  auto zero_rows = [&](int64_t from, int64_t to, int who, int n) {  // rows [from, to), n lanes
+    float* d = out + from * R;
+    const int64_t count = (to - from) * R;
+    if constexpr (VW % 4 == 0) {
+#pragma unroll 1
+      for (int64_t i = who; 4 * i < count; i += n)
+        reinterpret_cast<float4*>(d)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
+#pragma unroll 1
+      for (int64_t i = who; i < count; i += n) d[i] = 0.f;
+    }
+  };
+  // All lanes: the row `cur` ends: to the block's partials where it is split, else to
+  // M_n after the empty rows before it (and, for the mode's last row, those after it).
+  auto close_row = [&](int stage, bool last) {
+    float* to = out + (int64_t)cur * R;
+    float s = sc;
+    bool trail = false;
+    if (first || last || prev + 1 < cur) {
+      const int4 d = desc[stage];
+      const int fl = d.y >> 16;
+      if ((first && (fl & BLK_HEAD_SPLIT)) || (last && (fl & BLK_TAIL_SPLIT))) {
+        to = a.part + ((size_t)d.z * 2 + (first ? 0 : 1)) * R;
+        s = 1.f;
+      } else if (!a.no_fill) {
+        if (prev + 1 < cur) zero_rows((int64_t)prev + 1, cur, lane, 32);
+        trail = last && cur == a.last_row;
+      }
+      first = false;
+    }
+#pragma unroll 1
+    for (int o = L; o < 32; o <<= 1)
+#pragma unroll
+      for (int j = 0; j < NV; ++j) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+    if (gw == 0) store_row(to, acc, s);
+    if (trail) zero_rows((int64_t)cur + 1, a.out_rows, lane, 32);
+  };
+  // Adds the n nonzeros whose weighted products lie in the scratch (staged from p0 on)
+  // to their rows.
+  auto add_rows = [&](int n, const uint8_t* p0, int stage) {
+    __syncwarp();
+#pragma unroll 1
+    for (int b = 0; b < n; b += 32) {
+      const int m = min(32, n - b);
+      const int row = lane < m ? row_of(p0 + (b + lane) * es) : -1;
+      int before = __shfl_up_sync(0xffffffffu, row, 1);
+      if (lane == 0) before = cur;
+      const unsigned starts = __ballot_sync(0xffffffffu, lane < m && row != before);
+      const int nst = __popc(starts);
+      // slot i of the list: where the batch's i-th new row begins; then its end
+      if ((starts >> lane) & 1u) srows[__popc(starts & ((1u << lane) - 1u))] = lane;
+      if (lane == 0) srows[nst] = m;
+      __syncwarp();
+      int j = 0, e = srows[0];
+#pragma unroll 1
+      while (true) {  // first the row `cur` up to its end, then the batch's last row
+#pragma unroll 2
+        for (int k = j + gw; k < e; k += G) add_slot(b + k, acc);
+        if (nst == 0 || e == m) break;
+        close_row(stage, false);
+        prev = cur;
+        // the rows between, a group each
+        if (nst > 1) {
+#pragma unroll 1
+          for (int i = gw; i < nst - 1; i += G) {
+            const int k0 = srows[i], k1 = srows[i + 1];
+            const uint8_t* p = p0 + (b + k0) * es;
+            const int r = row_of(p), rb = i > 0 ? row_of(p - es) : cur;
+            float v[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q) v[q] = 0.f;
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k) add_slot(b + k, v);
+            if (!a.no_fill && rb + 1 < r) zero_rows((int64_t)rb + 1, r, sub, L);
+            store_row(out + (int64_t)r * R, v, sc);
+          }
+          __syncwarp();
+          prev = row_of(p0 + (b + srows[nst - 1] - 1) * es);
+        }
+        j = srows[nst - 1];
+        e = m;
+        cur = row_of(p0 + (b + j) * es);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) acc[q] = 0.f;
+      }
+      __syncwarp();
+    }
+  };
+  double lsum = 0.0;  // LOSS: sum of squared residuals (FP32 per chunk, FP64 across)
+  auto end_block = [&](int stage) {
+    close_row(stage, true);
+    if constexpr (LOSS) {  // fixed-order warp sum of the lanes' partials
+      for (int off = 16; off > 0; off >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, off);
+      if (lane == 0) a.loss_part[desc[stage].z] = lsum;
+      lsum = 0.0;
+    }
+  };
+
+  // ---- the walk: chunks of U steps of G nonzeros (nonzero u G + g of the chunk is
+  // step u of group g), a rolling ring of one chunk per warp.  While a chunk is
+  // consumed, step after step, each step's place in the ring is filled at once with
+  // the gathers of the same step of the next chunk, across tile and block ends, so the
+  // warp always has close to U G nonzeros' rows in flight and never drains.
+  const int CH = U * G;
+  constexpr int NI = (NT > 0 ? NT : 2) - 1;
+  using P = Piece<T, VW>;
+  typename P::type raw[U][NI][RC];
+  typename P::type rown[LOSS ? U : 1][RC];  // A_n[i_n] (fused loss)
+  // this lane's pieces of the factor rows (pieces past R read piece 0 of the row;
+  // their values are never stored)
+  const uint8_t* base[NI];
+  const uint8_t* own = nullptr;
+  uint32_t poff[RC];
+#pragma unroll
+  for (int j = 0; j < RC; ++j)
+    poff[j] = (piece_rank(j) < R ? (uint32_t)piece_rank(j) : 0u) * (uint32_t)sizeof(T);
+#pragma unroll
+  for (int j = 0; j < NI; ++j) {
+    int k = mode + 1 + j;
+    if (k >= N) k -= N;
+    base[j] = static_cast<const uint8_t*>(a.factors[k]) + (RC == 1 ? poff[0] : 0u);
+  }
+  if constexpr (LOSS) own = static_cast<const uint8_t*>(a.factors[mode]) + poff[0];
+  const bool lane_live = sub * VW < R;
+
+  auto val_of = [&](const uint8_t* ep) -> float {
+    if constexpr (NT == 0) return elem_value(ep, N, a.pk);
+    else return reinterpret_cast<const float*>(ep)[PK ? 3 : NT];
+  };
+  // the rows to gather of the staged nonzero at ep (LOSS: its own row too)
+  auto fetch = [&](const uint8_t* ep, int& row, int (&ix)[NI]) {
+    if constexpr (NT == 3 && MODE >= 0) {
+      const int4 v = *reinterpret_cast<const int4*>(ep);
+      const int f[3] = {v.x, v.y, v.z};
+      row = f[MODE];
+      ix[0] = f[(MODE + 1) % 3];
+      ix[1] = f[(MODE + 2) % 3];
+    } else if constexpr (PK) {  // 4-6 modes in 16 bytes (bit fields)
+      const uint4 w4 = *reinterpret_cast<const uint4*>(ep);
+      const uint32_t w[3] = {w4.x, w4.y, w4.z};
 #pragma unroll
       for (int j = 0; j < NI; ++j) {
-        if (j < N - 1) {
-          const int kj = (NT == 3 && MODE >= 0) ? (MODE + 1 + j) % 3 : (mode + 1 + j) % N;
-          const void* Ak = a.factors[kj];
+        int k = mode + 1 + j;
+        if (k >= N) k -= N;
+        ix[j] = (int)pk_field(w, a.pk.off[k], a.pk.bits[k]);
+      }
+    } else if constexpr (NT > 0) {
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (u < nb) Landing<T, VW, RC>::load(Ak, ixs[u][j], R, sub, L, pol_factor, raw[u][j]);
-        }
+      for (int j = 0; j < NI; ++j) ix[j] = *reinterpret_cast<const int*>(ep + foff[1 + j]);
+    }
+  };
+  auto gather = [&](int u, int row, const int (&ix)[NI]) {
+    if constexpr (LOSS) {
+      const uint8_t* r = own + (uint64_t)(uint32_t)row * rowb;
+#pragma unroll
+      for (int q = 0; q < RC; ++q) rown[u][q] = P::load(r, pol_factor);
+    }
+#pragma unroll
+    for (int j = 0; j < NI; ++j) {  // one 32 x 32 -> 64-bit multiply-add per row address
+      const uint8_t* r = base[j] + (uint64_t)(uint32_t)ix[j] * rowb;
+#pragma unroll
+      for (int q = 0; q < RC; ++q) raw[u][j][q] = P::load(RC == 1 ? r : r + poff[q], pol_factor);
+    }
+  };
+  auto product = [&](int u, float (&prod)[NV]) {  // of the gathered pieces, in mode order
+#pragma unroll
+    for (int q = 0; q < RC; ++q) P::unpack(raw[u][0][q], prod + q * VW);
+#pragma unroll
+    for (int j = 1; j < NI; ++j) {
+      float x[NV];
+#pragma unroll
+      for (int q = 0; q < RC; ++q) P::unpack(raw[u][j][q], x + q * VW);
+      if constexpr (NV % 2 == 0) {  // paired FP32: half the instructions
+        float2* p2 = reinterpret_cast<float2*>(prod);
+        const float2* x2 = reinterpret_cast<const float2*>(x);
+#pragma unroll
+        for (int q = 0; q < NV / 2; ++q) p2[q] = mul2(p2[q], x2[q]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) prod[q] *= x[q];
       }
     }
-    if constexpr (LOSS) {
-      // the residual of each nonzero: m_e = sum over the lanes of the group of
-      // sum_q A_k1 A_k2 A_n, then e = m_e - x_e replaces the value
-      float m[U];
+  };
+  auto accumulate = [&](const float (&prod)[NV], float v) {
+    if constexpr (NV % 2 == 0) {
+      float2* a2 = reinterpret_cast<float2*>(acc);
+      const float2* p2 = reinterpret_cast<const float2*>(prod);
+      const float2 vv = make_float2(v, v);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        m[u] = 0.f;
-        if (u < nb) {
-          float p[NV], x[NV], y[NV];
-          Landing<T, VW, RC>::unpack(raw[u][0], p);
-          Landing<T, VW, RC>::unpack(raw[u][1], x);
-          Landing<T, VW, RC>::unpack(rown[u], y);
+      for (int q = 0; q < NV / 2; ++q) a2[q] = fma2(p2[q], vv, a2[q]);
+    } else {
 #pragma unroll
-          for (int q = 0; q < NV; ++q) {
-            hh[u][q] = p[q] * x[q];  // kept: the gradient's product below
-            m[u] = fmaf(hh[u][q], y[q], m[u]);
-          }
-          if (!lane_live) m[u] = 0.f;
-        }
+      for (int q = 0; q < NV; ++q) acc[q] = fmaf(prod[q], v, acc[q]);
+    }
+  };
+  // A chunk consumed (nc nonzeros, staged from pc on) while the next one (nn, staged
+  // from pn on) is gathered into its places of the ring.  The fast body takes a whole
+  // chunk inside one output row, the slow one any chunk; which of them depends on the
+  // block alone, never on what the warp takes next, so results do not depend on the
+  // claims.  Each step reads the fields of the next one ahead of its own arithmetic;
+  // the empty asm keeps the compiler from reading all steps' fields at once (the ring
+  // holds most of the registers).
+  const int gs = G * es;  // bytes from a group's nonzero to its next
+  auto body_fast = [&](auto full, int nn, const uint8_t* pc, const uint8_t* pn) {
+    constexpr bool FULL = decltype(full)::value;  // the next chunk is whole too
+    const uint8_t* ec = pc + gw * es;  // this group's nonzero of the step
+    const uint8_t* en = pn + gw * es;  // and of the next chunk's step
+    int nrow = 0, nix[NI];
+#pragma unroll
+    for (int j = 0; j < NI; ++j) nix[j] = 0;
+    if (FULL || gw < nn) fetch(en, nrow, nix);
+    float nval = val_of(ec);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      int ix_g[NI];
+#pragma unroll
+      for (int j = 0; j < NI; ++j) ix_g[j] = nix[j];
+      const float v = nval;
+      if (u + 1 < U) {
+        en += gs;
+        ec += gs;
+        if (FULL || (u + 1) * G + gw < nn) fetch(en, nrow, nix);
+        nval = val_of(ec);
+        asm volatile("" ::: "memory");  // read here, a step before they are used
       }
-      // the group's lanes run together (their segment lengths agree), other
-      // groups may be on another batch size: shuffle within the group only
-      const unsigned gmask = L >= 32 ? 0xffffffffu : (((1u << L) - 1u) << (gw * L));
-      if constexpr (U == 4) {
-        if (L >= 4) {
-          group_sum4(m, sub, L, gmask);
-        } else {
+      float prod[NV];
+      product(u, prod);
+      accumulate(prod, v);
+      if (FULL || u * G + gw < nn) gather(u, 0, ix_g);
+      asm volatile("" ::: "memory");
+    }
+  };
+  auto body_slow = [&](int nc, int nn, const uint8_t* pc, const uint8_t* pn, int stage) {
+    int i = gw;
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            for (int off = L / 2; off > 0; off >>= 1) m[u] += __shfl_xor_sync(gmask, m[u], off);
-        }
+    for (int u = 0; u < U; ++u, i += G) {
+      int nrow = 0, nix[NI];
+#pragma unroll
+      for (int j = 0; j < NI; ++j) nix[j] = 0;
+      if (i < nn) fetch(pn + i * es, nrow, nix);
+      const float v = i < nc ? val_of(pc + i * es) : 0.f;
+      float prod[NV];
+      product(u, prod);
+      if (i < nc) store_row(scratch + ((u % HS) * G + gw) * R, prod, v);
+      if (i < nn) gather(u, nrow, nix);
+      if (u % HS == HS - 1) {
+        const int u0 = (u - HS + 1) * G;
+        if (u0 < nc) add_rows(min(nc - u0, HS * G), pc + u0 * es, stage);
+      }
+      asm volatile("" ::: "memory");
+    }
+  };
+  // The fused CP-loss pass: the chunk's model values first (their products kept for the
+  // gradient), the next chunk's gathers behind them, then the residuals and the rows.
+  auto body_loss = [&](bool fast, int nc, int nn, uint8_t* pc, const uint8_t* pn, int stage) {
+    float m[U], hh[U][NV];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = u * G + gw;
+      int nrow = 0, nix[NI];
+#pragma unroll
+      for (int j = 0; j < NI; ++j) nix[j] = 0;
+      if (i < nn) fetch(pn + i * es, nrow, nix);
+      // the model value: m_e = sum over the lanes of the group of sum_q A_k1 A_k2 A_n
+      float y[NV];
+      product(u, hh[u]);
+      P::unpack(rown[u][0], y);
+      m[u] = 0.f;
+#pragma unroll
+      for (int q = 0; q < NV; ++q) m[u] = fmaf(hh[u][q], y[q], m[u]);
+      if (!lane_live || i >= nc) m[u] = 0.f;
+      if (i < nn) gather(u, nrow, nix);
+      asm volatile("" ::: "memory");
+    }
+    if constexpr (U == 4) {  // (always, where this pass is built)
+      // shuffles within the group's lanes
+      if (L >= 4) {
+        group_sum4(m, sub, L, 0xffffffffu);
       } else {
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          for (int off = L / 2; off > 0; off >>= 1) m[u] += __shfl_xor_sync(gmask, m[u], off);
+          for (int o = L / 2; o > 0; o >>= 1) m[u] += __shfl_xor_sync(0xffffffffu, m[u], o);
       }
-      float sq = 0.f;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u < nb) {
-          const float r = m[u] - vals[u];
-          vals[u] = r;
-          sq = fmaf(r, r, sq);
-          if (sub == 0)  // the residual copy: the staged nonzero's value becomes e
-            reinterpret_cast<float*>(const_cast<uint8_t*>(eb) + (size_t)(e + u) * es)[3] = r;
-        }
-      }
-      if (sub == 0) lsum += (double)sq;
     }
-    // rows are sorted within a run: if the batch's last nonzero is still in the
-    // current row, every nonzero of the batch is, and no per-nonzero check is needed
-    bool same_row = true;
+    float sq = 0.f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = u * G + gw;
+      if (i < nc) {  // the residual e = m_e - x_e replaces the value
+        m[u] -= val_of(pc + i * es);
+        sq = fmaf(m[u], m[u], sq);
+      }
+    }
+    if (sub == 0) lsum += (double)sq;
+    __syncwarp();  // every lane has read the chunk's values
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = u * G + gw;
+      if (sub == 0 && i < nc)  // the residual copy: the staged value becomes e
+        reinterpret_cast<float*>(pc + i * es)[3] = m[u];
+      if (fast) accumulate(hh[u], m[u]);
+    }
+    if (fast) return;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = u * G + gw;
+      if (i < nc) store_row(scratch + ((u % HS) * G + gw) * R, hh[u], m[u]);
+      if (u % HS == HS - 1) {
+        const int u0 = (u - HS + 1) * G;
+        if (u0 < nc) add_rows(min(nc - u0, HS * G), pc + u0 * es, stage);
+      }
+    }
+  };
+  // Runtime number of modes: a chunk's nonzeros are gathered mode by mode when it is
+  // consumed, each slice multiplied in as it lands.
+  auto body_generic = [&](int nc, const uint8_t* pc, int stage) {
+    float pr[U][NV];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (u == nb - 1) same_row = (rows[u] == cur);
-    if (same_row) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u < nb) {
-          float prod[NV], x[NV];
-          if constexpr (LOSS) {
-#pragma unroll
-            for (int q = 0; q < NV; ++q) prod[q] = hh[u][q];
-          } else {
-            Landing<T, VW, RC>::unpack(raw[u][0], prod);
-          }
-          if constexpr (NV % 2 == 0) {  // paired FP32: half the instructions
-            float2* p2 = reinterpret_cast<float2*>(prod);
-            if constexpr (!LOSS) {
-#pragma unroll
-              for (int j = 1; j < NI; ++j) {
-                if (j < N - 1) {
-                  Landing<T, VW, RC>::unpack(raw[u][j], x);
-                  const float2* x2 = reinterpret_cast<const float2*>(x);
-#pragma unroll
-                  for (int q = 0; q < NV / 2; ++q) p2[q] = mul2(p2[q], x2[q]);
-                }
-              }
-            }
-            float2* a2 = reinterpret_cast<float2*>(acc);
-            const float2 vv = make_float2(vals[u], vals[u]);
-#pragma unroll
-            for (int q = 0; q < NV / 2; ++q) a2[q] = fma2(p2[q], vv, a2[q]);
-          } else {
-            if constexpr (!LOSS) {
-#pragma unroll
-              for (int j = 1; j < NI; ++j) {
-                if (j < N - 1) {
-                  Landing<T, VW, RC>::unpack(raw[u][j], x);
-#pragma unroll
-                  for (int q = 0; q < NV; ++q) prod[q] *= x[q];
-                }
-              }
-            }
-#pragma unroll
-            for (int q = 0; q < NV; ++q) acc[q] = fmaf(prod[q], vals[u], acc[q]);
-          }
-        }
-      }
-      return;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (u < nb) {
-        float prod[NV], x[NV];
-        if constexpr (LOSS) {
-#pragma unroll
-          for (int q = 0; q < NV; ++q) prod[q] = hh[u][q];
-        } else {
-          Landing<T, VW, RC>::unpack(raw[u][0], prod);
-#pragma unroll
-          for (int j = 1; j < NI; ++j) {
-            if (j < N - 1) {
-              Landing<T, VW, RC>::unpack(raw[u][j], x);
-#pragma unroll
-              for (int q = 0; q < NV; ++q) prod[q] *= x[q];
-            }
-          }
-        }
-        if (rows[u] != cur) {
-          if constexpr (VW > 1 && RC == 1 && NT >= 3 && NT <= 5) {  // (6 modes: more spills)
-            RowAcc<NV> ra;
-#pragma unroll
-            for (int q = 0; q < NV; ++q) ra.v[q] = acc[q];
-            const int2 st2 = close_row<NV>(ra, cur, prev_in_run, head ? 1 : 0, out, R, sub, sc,
-                                           a.last_row, out_rows, a.no_fill, 2 * gw, srow, sprev,
-                                           sacc);
-            prev_in_run = st2.x;
-            head = st2.y != 0;
-          } else {
-            if (head) {
-              if (cur >= 0) {
-                store_slot(2 * gw, cur, -2, acc);
-                head = false;
-              }
-            } else {
-              write_row_group(cur, acc, prev_in_run);
-            }
-            if (cur >= 0) prev_in_run = cur;
-          }
-          cur = rows[u];
-#pragma unroll
-          for (int q = 0; q < NV; ++q) acc[q] = 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < NV; ++q) acc[q] = fmaf(prod[q], vals[u], acc[q]);
-      }
-    }
-  };
-  // runtime number of modes: multiply each gathered slice in as it lands
-  auto batch_generic = [&](int e, int nb) {
-    float prod[U][NV];
-    float vals[U];
-    int rows[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (u < nb) {
-        const uint8_t* ep = eb + (size_t)(e + u) * es;
-        rows[u] = elem_index(ep, mode, a.pk);
-        vals[u] = elem_value(ep, N, a.pk);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) prod[u][q] = vals[u];
-      }
-    }
+      for (int j = 0; j < NV; ++j) pr[u][j] = 1.f;
     for (int k = 0; k < N; ++k) {
       if (k == mode) continue;
-      const void* Ak = a.factors[k];
+      const uint8_t* Ak = static_cast<const uint8_t*>(a.factors[k]);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        if (u < nb) {
-          typename Landing<T, VW, RC>::type raw;
-          float x[NV];
-          Landing<T, VW, RC>::load(Ak, elem_index(eb + (size_t)(e + u) * es, k, a.pk), R, sub, L,
-                                   pol_factor, raw);
-          Landing<T, VW, RC>::unpack(raw, x);
+        if (u * G + gw >= nc) continue;
+        const uint8_t* r =
+            Ak + (uint64_t)(uint32_t)elem_index(pc + (u * G + gw) * es, k, a.pk) * rowb;
 #pragma unroll
-          for (int q = 0; q < NV; ++q) prod[u][q] *= x[q];
+        for (int j = 0; j < RC; ++j) {
+          float x[VW];
+          P::unpack(P::load(r + poff[j], pol_factor), x);
+#pragma unroll
+          for (int c = 0; c < VW; ++c) pr[u][j * VW + c] *= x[c];
         }
       }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (u < nb) {
-        if (rows[u] != cur) {
-          if (head) {
-            if (cur >= 0) {
-              store_slot(2 * gw, cur, -2, acc);
-              head = false;
-            }
-          } else {
-            write_row_group(cur, acc, prev_in_run);
-          }
-          if (cur >= 0) prev_in_run = cur;
-          cur = rows[u];
-#pragma unroll
-          for (int q = 0; q < NV; ++q) acc[q] = 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < NV; ++q) acc[q] += prod[u][q];
+      const int i = u * G + gw;
+      if (i < nc) store_row(scratch + ((u % HS) * G + gw) * R, pr[u], val_of(pc + i * es));
+      if (u % HS == HS - 1) {
+        const int u0 = (u - HS + 1) * G;
+        if (u0 < nc) add_rows(min(nc - u0, HS * G), pc + u0 * es, stage);
       }
     }
   };
 
-  int issued = min(ntiles, S - 1);
-  for (int t = 0; t < ntiles; ++t) {
-    const int st = t % S;
-    // the stall test waits first on mbar[S], which no copy and no thread completes
-    const bool stall = a.stall_test && t == 0;
-    const bool ok = mbar_wait_bounded(stall ? &mbar[S] : &mbar[st],
-                                      stall ? 0u : (uint32_t)((t / S) & 1), wait_ns);
-    if (!__all_sync(0xffffffffu, ok)) {
-      // a bulk copy did not complete in time: record it, wait (bounded) for
-      // the copies still in flight, and leave without writing anything else
-      if (lane == 0) {
-        atomicOr(a.err, 1);
-        for (int q = t; q < issued; ++q)
-          (void)mbar_wait_bounded(&mbar[q % S], (uint32_t)((q / S) & 1));
+  if (!wait_tile(0, 0)) return;
+  int stage = 0;        // the gathering side's tile: its stage, the phase of its barrier,
+  uint32_t phase = 0;   // its flags, and its nonzeros not yet gathered
+  int dy = desc[0].y, left = dy & 0xffff;
+  if (left == 0) return;  // the warp has no nonzeros
+  if (remap && !LOSS) do_remap(0);
+  uint8_t* pn = ebuf;
+  int nn = min(CH, left);
+  if constexpr (NT > 0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (u * G + gw < nn) {
+        int row = 0, nix[NI];
+        fetch(pn + (u * G + gw) * es, row, nix);
+        gather(u, row, nix);
       }
-      return;
     }
-    // the stage of tile t+S-1 held tile t-1, whose readers passed the last __syncwarp
-    if (leader && t + S - 1 < ntiles) issue(t + S - 1);
-    issued = min(ntiles, t + S);
-    const int seg = ga + t * K;
-    const int n = max(0, min(K, gb - seg));
-    eb = ebuf + ((size_t)st * TW + (size_t)gw * K) * es;
-
-    auto do_remap = [&]() {  // Algorithm 3: every element to its place in the next mode's order
-      const int32_t* np = npbuf + (st * G + gw) * NPK + (seg & 3);
-      if (es % 32 == 0) {  // whole 32-byte sectors per store (no read of the old sector)
-        const int nv = es >= 32 ? es / 32 : 1;
-        const int aw = a.alpha_word;  // remap id carried in the staged nonzero (Section 3.5)
-        for (int i = sub; i < n * nv; i += L) {
-          const int e = (nv == 1) ? i : i / nv, c = (nv == 1) ? 0 : i - e * nv;
-          const uint4* src = reinterpret_cast<const uint4*>(eb + (size_t)e * es) + 2 * c;
-          const uint4 lo = src[0], hi = src[1];
-          // with the ids in the nonzero (32-byte stride, one sector: c == 0) the id is
-          // word aw of the sector, i.e. component aw - 4 of its upper half
-          // (bit 31 of the id words is a hot-row flag, not part of the id)
-          const int dst = aw ? (int)((aw == 4 ? hi.x : (aw == 5 ? hi.y : hi.z)) & 0x7fffffffu)
-                             : np[e];
-          st_hint_v8(a.elems_out + (size_t)dst * es + 32 * c, lo, hi, pol_stream);
-        }
-      } else {
-        const int nv = es / 16;  // 16-byte vectors per element (constant when NT > 0)
-        for (int i = sub; i < n * nv; i += L) {
-          const int e = (nv == 1) ? i : i / nv, c = (nv == 1) ? 0 : i - e * nv;
-          const uint4 v = reinterpret_cast<const uint4*>(eb + (size_t)e * es)[c];
-          st_hint_v4(reinterpret_cast<uint4*>(a.elems_out + (size_t)np[e] * es) + c, v,
-                     pol_stream);
-        }
+  }
+  bool block_start = true;
+  const int last_off = (CH - 1) * es;
+#pragma unroll 1
+  while (nn > 0) {
+    uint8_t* pc = pn;  // the chunk to consume
+    const int nc = nn, cstage = stage;
+    left -= nn;
+    const bool tile_end = left == 0;
+    bool block_end = false;
+    if (tile_end) {
+      block_end = ((dy >> 16) & kLast) != 0;
+      if (++stage == S) {
+        stage = 0;
+        phase ^= 1u;
       }
-    };
-    if (remap && !LOSS) do_remap();
-
-    // Algorithm 2 over this group's segment [0, n) of the tile
-    int e = 0;
-    if constexpr (NT > 0) {
-      for (; e + U <= n; e += U) batch(e, U);
-      for (; e < n; ++e) batch(e, 1);
+      if (!wait_tile(stage, phase)) return;
+      dy = desc[stage].y;
+      left = dy & 0xffff;
+      if (remap && !LOSS && left > 0) do_remap(stage);
+      pn = ebuf + (size_t)stage * TW * es;
     } else {
-      for (; e + U <= n; e += U) batch_generic(e, U);
-      for (; e < n; ++e) batch_generic(e, 1);
+      pn += CH * es;
     }
-    if constexpr (LOSS) {  // the residual nonzeros, now in shared memory, to the next order
+    nn = min(CH, left);
+    if (block_start) {
+      prev = desc[cstage].w;
+      cur = row_of(pc);
+      first = true;
+#pragma unroll
+      for (int j = 0; j < NV; ++j) acc[j] = 0.f;
+      block_start = false;
+    }
+    if constexpr (NT == 0) {
+      body_generic(nc, pc, cstage);
+    } else {
+      const bool fast = nc == CH && row_of(pc + last_off) == cur;
+      if constexpr (LOSS) body_loss(fast, nc, nn, pc, pn, cstage);
+      else if (fast && nn == CH) body_fast(std::true_type{}, nn, pc, pn);
+      else if (fast) body_fast(std::false_type{}, nn, pc, pn);
+      else body_slow(nc, nn, pc, pn, cstage);
+    }
+    if (tile_end) {  // the consumed chunk was its tile's last: the tile's stage is free
       __syncwarp();
-      if (remap) do_remap();
-    }
-    __syncwarp();
-  }
-
-  // the run's first row (head) and last row (tail) as partial sums
-  if (cur < 0) {  // empty run
-    if (sub == 0) {
-      srow[2 * gw] = -1;
-      srow[2 * gw + 1] = -1;
-    }
-  } else if (head) {
-    store_slot(2 * gw, cur, -2, acc);
-    if (sub == 0) srow[2 * gw + 1] = -1;
-  } else {
-    store_slot(2 * gw + 1, cur, prev_in_run, acc);
-  }
-  __syncwarp();
-
-  // warp combine: run-boundary rows in run order, then the block's last row
-  int crow = -1, cprev = bi.z, emitted = 0;
-  auto emit = [&](int row, int prev, bool first, bool last) {
-    const bool split = (first && (bi.w & BLK_HEAD_SPLIT)) || (last && (bi.w & BLK_TAIL_SPLIT));
-    if (split) {
-      float* d = a.part + ((size_t)wb * 2 + (first ? 0 : 1)) * R;
-      for (int r = lane; r < R; r += 32) d[r] = cacc[r];
-      return;
-    }
-    for (int64_t z = a.no_fill ? (int64_t)row : (int64_t)prev + 1; z < row; ++z)
-      for (int r = lane; r < R; r += 32) out[z * R + r] = 0.f;
-    for (int r = lane; r < R; r += 32) out[(int64_t)row * R + r] = cacc[r] * sc;
-    if (!a.no_fill && row == a.last_row)
-      for (int64_t z = (int64_t)row + 1; z < out_rows; ++z)
-        for (int r = lane; r < R; r += 32) out[z * R + r] = 0.f;
-  };
-  for (int s = 0; s < 2 * G; ++s) {
-    const int row = srow[s];
-    if (row < 0) continue;
-    const float* sa = sacc + (size_t)s * R;
-    if (row == crow) {
-      for (int r = lane; r < R; r += 32) cacc[r] += sa[r];
-    } else {
-      if (crow >= 0) {
-        emit(crow, cprev, emitted == 0, false);
-        emitted = 1;
+      if (LOSS && remap) {  // the residual nonzeros, now in shared memory, to the next order
+        do_remap(cstage);
+        __syncwarp();
       }
-      const int pv = sprev[s];
-      cprev = (pv != -2) ? pv : (crow >= 0 ? crow : cprev);
-      crow = row;
-      for (int r = lane; r < R; r += 32) cacc[r] = sa[r];
+      if (block_end) {
+        end_block(cstage);
+        block_start = true;
+        __syncwarp();
+      }
+      issue(cstage);
     }
-    __syncwarp();
-  }
-  if (crow >= 0) emit(crow, cprev, emitted == 0, true);
-  if constexpr (LOSS) {  // fixed-order warp sum of the lanes' partials
-    for (int off = 16; off > 0; off >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, off);
-    if (lane == 0) a.loss_part[wb] = lsum;
   }
 }
 
-// Nonzeros per warp tile for a requested size: G runs of an odd length K, so
-// that the groups' elements fall on distinct shared-memory banks.
-__host__ __device__ inline int warp_tile_for(int tile, int G) {
-  int K = tile / G;
-  if (K < 1) K = 1;
-  if (!(K & 1)) K += 1;
-  return G * K;
+// Nonzeros per warp tile for a requested size: a whole number of chunks (U steps
+// of G nonzeros).
+__host__ __device__ inline int warp_tile_for(int tile, int G, int U) {
+  const int c = G * U;
+  return c * (tile / c > 1 ? tile / c : 1);
 }
+
+// CTAs of the fused kernel that are resident at once on the current device with
+// `smem` bytes of dynamic shared memory each (asked once per kernel, size and device).
+int resident_ctas(const void* kernel, size_t smem, int* ctas);
 
 template <int NT, typename T, int VW, int RC, int U, int MODE = -1, int ESB = 0, bool LOSS = false,
-          bool RWARP = false>
+          bool RWARP = false, bool PK = false>
 int launch_warp_kernel(const MttkrpArgs& a0, int L, cudaStream_t s) {
   const int G = 32 / L;
   MttkrpArgs a = a0;
-  a.tile = warp_tile_for(a0.tile, G);
+  // (form 3's remap warp leaves its CTA less room)
+  a.tile = warp_tile_for(RWARP ? std::min(a0.tile, 64) : a0.tile, G, U);
+  constexpr int CW = RWARP ? kWarps - 1 : kWarps;  // warps that compute
   // form 3: seven compute warps' slots, then the remap warp's region
-  const size_t smem = RWARP ? (size_t)(kWarps - 1) * warp_layout(a.es, a.tile, a.R, G, a.stages).total +
-                                  kRemapRegion
-                            : (size_t)kWarps * warp_layout(a.es, a.tile, a.R, G, a.stages).total;
-  auto kfn = mttkrp_warp_kernel<NT, T, VW, RC, U, MODE, ESB, LOSS, RWARP>;
+  const size_t smem = CW * warp_layout(a.es, a.tile, a.stages, a.alpha_word == 0).total +
+                      (RWARP ? kRemapRegion : 0);
+  auto kfn = mttkrp_warp_kernel<NT, T, VW, RC, U, MODE, ESB, LOSS, RWARP, PK>;
   int st = ensure_dyn_smem((const void*)kfn, smem, "cudaFuncSetAttribute(mttkrp_warp)");
   if (st) return st;
-  constexpr int CW = RWARP ? kWarps - 1 : kWarps;  // blocks per CTA
-  const int grid = (a.nblk + CW - 1) / CW;
+  int grid = (a.nblk + CW - 1) / CW;
+  if (!RWARP) {  // (form 3's remap warps cover their CTA's own blocks)
+    int ctas = 0;
+    st = resident_ctas((const void*)kfn, smem, &ctas);
+    if (st) return st;
+    grid = std::min(grid, ctas);
+    // blocks past the warps' first two are claimed from a counter
+    if (a.nblk > 2 * grid * CW) SPM_CUDA(cudaMemsetAsync(a.sched, 0, sizeof(int), s));
+  }
   kfn<<<grid, kThreads, smem, s>>>(a, L);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "mttkrp_warp_kernel launch");
   return SPM_OK;
 }
+
+// 4 to 6 modes: nonzeros in 32-byte sectors, or packed in 16 bytes.
+template <int NT, typename T, int VW, int U>
+int launch_modes(const MttkrpArgs& a, int L, cudaStream_t s) {
+  if (a.pk.packed) return launch_warp_kernel<NT, T, VW, 1, U, -1, 0, false, false, true>(a, L, s);
+  return launch_warp_kernel<NT, T, VW, 1, U>(a, L, s);
+}
+
+// Lanes of one or two values (ranks that are no multiple of four, or factors aligned
+// to less than 16 bytes): built for 3 to 6 modes and up to 64 columns; other shapes run
+// the runtime-modes kernel.
+inline bool narrow_built(const MttkrpArgs& a, const LaneCfg& c) {
+  return a.nmodes >= 3 && a.nmodes <= 6 && !a.pk.packed && c.VW * c.RC <= 2;
+}
+int launch_narrow_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s);
+int launch_narrow_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s);
 
 }  // namespace spm

@@ -101,11 +101,14 @@ int default_nblk(int64_t nnz, int num_sms, int variant) {
   if (nnz <= 0) return 1;
   int64_t nb;
   if (variant == 0 || variant == 3) {
-    // warp blocks (forms 0 and 3): about 16 waves of 24 warps per SM, each block >= 256
-    // nonzeros, and never more than 4K nonzeros per block (measured: blocks of
-    // 1.7-4K nonzeros sweep fastest on 60M-200M nonzero tensors)
-    nb = std::max<int64_t>(std::min<int64_t>((int64_t)num_sms * 24 * 16, (nnz + 255) / 256),
-                           (nnz + 4095) / 4096);
+    // warp blocks (forms 0 and 3), taken in order by the resident warps.  From 10M
+    // nonzeros on they hold 512 (the remap's stores then stay within what L2 holds: a
+    // 30M-nonzero sweep takes 2.28 ms with 512 and 2.37 with 1024; 256 pay more for
+    // their ends, 2.30), up to 1024 blocks per SM (larger blocks beyond: at 100M, 640
+    // and 1024 measure the same).  Below, 256, so that every warp has several to take.
+    const int64_t sms = num_sms;
+    nb = std::max(std::min((nnz + 255) / 256, sms * 128), std::min((nnz + 511) / 512, sms * 1024));
+    nb = std::max(nb, (nnz + 4095) / 4096);
   } else if (variant == 2) {
     // tile form: about 16 blocks per SM, taken dynamically by the persistent
     // CTAs, each at least four 960-nonzero tiles long
@@ -119,15 +122,9 @@ int default_nblk(int64_t nnz, int num_sms, int variant) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(nb, 1 << 22));
 }
 
-// Nonzeros per warp tile (the plan halves it while two 8-warp CTAs per SM would
-// not fit in shared memory: a 3-stage ring of 128 32-byte nonzeros per warp
-// would leave room for one, a 2-stage ring for two).
-int default_tile(int) { return 128; }
-
-// Position -> index of the nonempty row holding it (ustart ascending, size nu+1).
-static inline int64_t row_index_of(const std::vector<int64_t>& ustart, int64_t pos) {
-  return (int64_t)(std::upper_bound(ustart.begin(), ustart.end(), pos) - ustart.begin()) - 1;
-}
+// Nonzeros per warp tile: 2 KB of staged nonzeros per ring stage (the staging is taken
+// from the L1 the gathers land in; mttkrp_kernel.cuh has both sides measured).
+int default_tile(int es) { return es >= 32 ? 64 : 128; }
 
 // Algorithm 1 (Section 3.4): the mode's vertices (output rows) in descending
 // degree, equal degrees in ascending index, each to the block holding the fewest
@@ -190,19 +187,36 @@ int partition_mode(const spmttkrp_plan* p, int n, int nblk, ModeHost* out) {
   const int64_t nnz = p->nnz;
   const std::vector<int64_t>& us = p->row_start[n];   // nonempty-row starts (+nnz)
   const std::vector<int64_t>& ur = p->row_start[p->N + n];  // nonempty-row ids
+  // Position -> index of the nonempty row holding it (starts ascending, nonempty + 1 of
+  // them); the positions looked up ascend, so each search goes on where the last ended.
+  struct Cursor {
+    const std::vector<int64_t>& us;
+    int64_t u = 0;
+    int64_t at(int64_t pos) {
+      int64_t step = 1;  // gallop, then search between
+      while (u + step + 1 < (int64_t)us.size() && us[(size_t)(u + step)] <= pos) {
+        u += step;
+        step *= 2;
+      }
+      const int64_t e = std::min<int64_t>(u + step + 1, (int64_t)us.size());
+      u = (int64_t)(std::upper_bound(us.begin() + u, us.begin() + e, pos) - us.begin()) - 1;
+      return u;
+    }
+  };
   ModeHost m;
   m.nblk = nblk;
   m.bounds.assign((size_t)nblk + 1, 0);
   m.bounds[nblk] = nnz;
   if (nnz > 0) {
     const int64_t T = (nnz + nblk - 1) / nblk;
+    Cursor c{us};
     for (int j = 1; j < nblk; ++j) {
       int64_t t = std::min<int64_t>((int64_t)j * T, nnz);
       if (t >= nnz) {
         m.bounds[j] = nnz;
         continue;
       }
-      int64_t u = row_index_of(us, t);
+      int64_t u = c.at(t);
       int64_t s = us[u], e = us[u + 1];
       if (t == s)
         m.bounds[j] = t;
@@ -215,6 +229,7 @@ int partition_mode(const spmttkrp_plan* p, int n, int nblk, ModeHost* out) {
   }
   // per-block descriptors
   m.blkinfo.assign((size_t)nblk * 4, 0);
+  Cursor c{us};  // (looks at lo - 1, lo and hi - 1 of each nonempty block)
   for (int b = 0; b < nblk; ++b) {
     int64_t lo = m.bounds[b], hi = m.bounds[b + 1];
     int32_t* bi = &m.blkinfo[(size_t)b * 4];
@@ -223,23 +238,26 @@ int partition_mode(const spmttkrp_plan* p, int n, int nblk, ModeHost* out) {
     bi[2] = -1;
     bi[3] = 0;
     if (lo < hi) {
-      int64_t ulo = row_index_of(us, lo);
+      const int64_t uprev = lo > 0 ? c.at(lo - 1) : -1;
+      const int64_t ulo = c.at(lo);
       if (lo > 0) {
-        int64_t uprev = row_index_of(us, lo - 1);
         bi[2] = (int32_t)ur[uprev];
         if (uprev == ulo) bi[3] |= BLK_HEAD_SPLIT;
       }
       if (hi < nnz) {
-        if (row_index_of(us, hi) == row_index_of(us, hi - 1)) bi[3] |= BLK_TAIL_SPLIT;
+        const int64_t ulast = c.at(hi - 1);
+        // (the next block looks at hi - 1 again: leave the cursor there)
+        if (us[(size_t)(ulast + 1)] > hi) bi[3] |= BLK_TAIL_SPLIT;
       }
     }
   }
   // split rows: a boundary strictly inside a row
   int64_t last_u = -1;
+  Cursor cs{us};
   for (int j = 1; j < nblk; ++j) {
     int64_t t = m.bounds[j];
     if (t <= 0 || t >= nnz) continue;
-    int64_t u = row_index_of(us, t);
+    int64_t u = cs.at(t);
     if (us[u] < t && t < us[u + 1] && u != last_u) {
       SplitRow sr;
       int64_t s = us[u], e = us[u + 1];
