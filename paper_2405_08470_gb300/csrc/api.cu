@@ -79,6 +79,11 @@ int upload_mode_tables(spmttkrp_plan* p, int n) {
     p->dev_bytes -= std::max<size_t>((size_t)d.nempty * sizeof(int32_t), 16);
     d.empty_rows = nullptr;
   }
+  if (d.gaps) {
+    cudaFree(d.gaps);
+    p->dev_bytes -= std::max<size_t>((size_t)d.ngap * sizeof(int2), 16);
+    d.gaps = nullptr;
+  }
   d.nblk = h.nblk;
   d.nsplit = (int)h.splits.size();
   d.nchunk = h.nchunk;
@@ -97,6 +102,15 @@ int upload_mode_tables(spmttkrp_plan* p, int n) {
     st = plan_dalloc(p, (void**)&d.empty_rows, (size_t)d.nempty * sizeof(int32_t));
     if (st) return st;
     SPM_CUDA(cudaMemcpyAsync(d.empty_rows, h.empty_rows.data(), (size_t)d.nempty * sizeof(int32_t),
+                             cudaMemcpyHostToDevice, p->stream));
+  }
+  d.ngap = (int)(h.gaps.size() / 2);
+  d.has_gaps = d.ngap > 0;
+  if (p->max_bytes) d.ngap = 0;  // under a memory cap no list: the output is zeroed first
+  if (d.ngap) {
+    st = plan_dalloc(p, (void**)&d.gaps, (size_t)d.ngap * sizeof(int2));
+    if (st) return st;
+    SPM_CUDA(cudaMemcpyAsync(d.gaps, h.gaps.data(), (size_t)d.ngap * sizeof(int2),
                              cudaMemcpyHostToDevice, p->stream));
   }
   // fix-up scratch: one R-float sum per chunk of a split row's blocks
@@ -248,10 +262,15 @@ int run_mode(spmttkrp_plan* p, int mode, const void* const* factors, float* out,
   if ((a.variant == 2 || a.variant == 3) && !p->worders) a.variant = 0;  // no write orders
   // the pass's elements carry their remap ids: word 4 + (next mode)
   a.alpha_word = p->alpha ? 4 + (mode + 1) % p->N : 0;
+  a.gaps = d.gaps;
+  a.ngap = d.ngap;
+  const bool warp_form = runs_warp_form(a);
+  if (warp_form && d.has_gaps && d.ngap == 0)
+    SPM_CUDA(cudaMemsetAsync(out, 0, (size_t)a.out_rows * p->R * sizeof(float), p->stream));
   int st = launch_mttkrp(a, p->stream);
   if (st) return st;
   st = launch_fixup(p->d_part, d.splits, d.nsplit, d.nchunk, p->d_fixsum, out, a.out_rows, p->R,
-                    scale, p->stream);
+                    scale, !warp_form, p->stream);
   if (st) return st;
   return launch_zero_listed_rows(out, d.empty_rows, d.nempty, p->R, p->stream);
 }
@@ -515,6 +534,7 @@ int spmttkrp_plan_destroy(spmttkrp_plan_t p) {
     dfree(d.blkinfo);
     dfree(d.splits);
     dfree(d.empty_rows);
+    dfree(d.gaps);
   }
   dfree(p->d_part);
   dfree(p->d_fixsum);

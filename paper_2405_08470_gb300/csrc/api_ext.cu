@@ -509,7 +509,7 @@ int spmttkrp_autotune(spmttkrp_plan_t p, const void* const* factors, float* cons
   // ordered by them): only the tile, ring depth and form are tuned then
   const bool fixed_blocks = p->partition == 1;
   // n_per_sm < 0: the plan's size-based default block count
-  const int nblk_default = default_nblk(p->nnz, p->num_sms, 0);
+  const int nblk_default = default_nblk(p->nnz, p->num_sms, 0, p->max_bytes > 0);
   auto nblk_for = [&](int n_per_sm) {
     if (fixed_blocks) return p->mh[0].nblk;
     return n_per_sm < 0 ? nblk_default : std::max(1, n_per_sm * p->num_sms);

@@ -47,6 +47,13 @@ struct SplitRow {
 };
 constexpr int kFixChunk = 256;  // blocks summed by one CTA of the fix-up's first pass
 
+// Empty output rows (forms 0 and 3) come from a list of their runs, in pieces of at most
+// kGapRows rows that all lane groups of the fused kernel share.  Zeroed by whoever wrote
+// the next nonempty row, as the other forms do, an unused range of 180K ids held one mode
+// of a 20M-nonzero 5-mode tensor for 3.3 ms (0.65 of them for its nonzeros), and the code
+// for it stood in every place where a row can end.
+constexpr int kGapRows = 64;
+
 // Host-side result of planning one mode.
 struct ModeHost {
   int nblk = 0;
@@ -55,6 +62,7 @@ struct ModeHost {
   std::vector<SplitRow> splits;    // ascending rows
   int nchunk = 0;                  // fix-up chunks over all split rows
   int last_row = -1;               // row of position nnz-1
+  std::vector<int32_t> gaps;       // pieces of the runs of empty rows: {from, to}
   // partition 1 (Algorithm 1): nonzeros per block and the rows with none
   std::vector<int64_t> lpt_load;
   std::vector<int32_t> empty_rows;
@@ -69,6 +77,9 @@ struct ModeDev {
   SplitRow* splits = nullptr;
   int32_t* empty_rows = nullptr;  // partition 1: rows of this mode with no nonzero
   int nempty = 0;
+  int2* gaps = nullptr;            // runs of empty rows, in pieces {from, to}
+  int ngap = 0;
+  bool has_gaps = false;  // the mode has empty rows (and no list of them when ngap is 0)
   int nchunk = 0;                  // fix-up chunks of this mode's split rows
   int32_t* next_pos = nullptr;  // nnz (+4 padding ints)
 };
@@ -205,7 +216,7 @@ int build_write_orders(spmttkrp_plan* p, uint8_t* elems);
 int build_hot_flags(spmttkrp_plan* p, uint8_t* elems);
 int default_tile(int es);
 int partition_mode(const spmttkrp_plan* p, int n, int nblk, ModeHost* out);
-int default_nblk(int64_t nnz, int num_sms, int variant);
+int default_nblk(int64_t nnz, int num_sms, int variant, bool capped);
 
 // ---- kernel launchers (kernels_*.cu) ----
 struct MttkrpArgs {
@@ -231,6 +242,8 @@ struct MttkrpArgs {
   int stages;              // tiles per warp ring of the staged form (2..4)
   int no_fill;             // 1: blocks own non-contiguous row sets (Algorithm 1), so
                            // no kernel writes the empty rows between its rows
+  const int2* gaps;        // forms 0 and 3: pieces of the runs of empty rows
+  int ngap;
   int alpha_word;          // > 0: int32 word of a stored nonzero holding its position in
                            // the next mode's order (the remap id carried in the
                            // element); 0: the next_pos array
@@ -249,11 +262,12 @@ struct MttkrpArgs {
                            // of the hot rows of factor k (3 modes, 32-byte nonzeros)
 };
 int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s);
+bool runs_warp_form(const MttkrpArgs& a);  // launch_mttkrp takes forms 0 or 3
 // the tile form (form 2) covers 3 modes, 32-byte nonzeros carrying remap ids, R 16/32/64
 bool tile_form_supported(int nmodes, int es, int alpha_word, int R);
 int launch_fixup(const float* part, const SplitRow* splits, int nsplit, int nchunk,
                  float* chunk_sums, float* out, int64_t out_rows, int R, const float* scale,
-                 cudaStream_t s);
+                 bool fill, cudaStream_t s);
 int launch_zero_rows(float* out, int64_t rows, int R, cudaStream_t s);
 int launch_zero_listed_rows(float* out, const int32_t* rows, int nrows, int R, cudaStream_t s);
 int launch_remap_only(const uint8_t* in, uint8_t* out, const int32_t* next_pos, int64_t nnz,

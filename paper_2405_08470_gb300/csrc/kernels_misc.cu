@@ -52,18 +52,26 @@ int resident_ctas(const void* kernel, size_t smem, int* ctas) {
   return SPM_OK;
 }
 
+// The tile form needs 16-byte aligned factors and output; otherwise form 0.
+static bool runs_tile_form(const MttkrpArgs& a) {
+  bool al = aligned16(a.out);
+  for (int k = 0; k < a.nmodes; ++k)
+    if (k != a.mode) al = al && aligned16(a.factors[k]);
+  return a.variant == 2 && !a.loss_part && al && a.no_fill == 0 &&
+         tile_form_supported(a.nmodes, a.es, a.alpha_word, a.R);
+}
+
+bool runs_warp_form(const MttkrpArgs& a) {
+  return a.loss_part || (a.variant != 1 && !runs_tile_form(a));
+}
+
 int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s) {
   if (a.nblk <= 0) return SPM_OK;
   LaneCfg c = cfg_for(a);
   if (a.loss_part)  // the fused CP-loss pass runs in the warp-block form
     return a.dtype == SPM_DTYPE_BF16 ? launch_mttkrp_bf16(a, c, s) : launch_mttkrp_f32(a, c, s);
   if (a.variant == 2) {
-    // the tile form needs 16-byte aligned factors and output; otherwise form 0
-    bool al = aligned16(a.out);
-    for (int k = 0; k < a.nmodes; ++k)
-      if (k != a.mode) al = al && aligned16(a.factors[k]);
-    if (al && tile_form_supported(a.nmodes, a.es, a.alpha_word, a.R) && a.no_fill == 0)
-      return launch_mttkrp_tile(a, s);
+    if (runs_tile_form(a)) return launch_mttkrp_tile(a, s);
     MttkrpArgs b = a;
     b.variant = 0;
     c = cfg_for(b);
@@ -85,7 +93,7 @@ int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s) {
 // bit-identical run to run).  Pass 1: one CTA per chunk of up to kFixChunk
 // consecutive blocks of a split row; warp w sums the chunk's blocks w, w+8, ...
 // (lanes over R) and the 8 warp sums are added in warp order.  Pass 2: one CTA
-// per split row adds its chunk sums in chunk order, writes the row once and
+// per split row adds its chunk sums in chunk order, writes the row once and (fill)
 // zeroes the empty rows before it (and after it, for the last nonempty row).  A
 // row spread over thousands of blocks (a Zipf head row) is summed by many CTAs.
 __global__ void __launch_bounds__(256) splitrow_chunk_kernel(const float* __restrict__ part,
@@ -127,14 +135,15 @@ __global__ void __launch_bounds__(256) splitrow_fixup_kernel(const float* __rest
                                                              const SplitRow* __restrict__ splits,
                                                              int nsplit, float* __restrict__ out,
                                                              int64_t out_rows, int R,
-                                                             const float* scale) {
+                                                             const float* scale, bool fill) {
   if ((int)blockIdx.x >= nsplit) return;
   const SplitRow sr = splits[blockIdx.x];
   const float sc = scale ? __ldg(scale) : 1.0f;
   const int nc = (sr.last_blk - sr.first_blk + kFixChunk) / kFixChunk;
   const int64_t gap0 = (int64_t)sr.prev_row + 1, ngap = ((int64_t)sr.row - gap0) * R;
-  for (int64_t i = threadIdx.x; i < ngap; i += blockDim.x) out[gap0 * R + i] = 0.f;
-  if (sr.is_last) {
+  if (fill)  // (forms 0 and 3 zero the empty rows from their list)
+    for (int64_t i = threadIdx.x; i < ngap; i += blockDim.x) out[gap0 * R + i] = 0.f;
+  if (fill && sr.is_last) {
     const int64_t t0 = (int64_t)sr.row + 1, nt = (out_rows - t0) * R;
     for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) out[t0 * R + i] = 0.f;
   }
@@ -147,11 +156,11 @@ __global__ void __launch_bounds__(256) splitrow_fixup_kernel(const float* __rest
 
 int launch_fixup(const float* part, const SplitRow* splits, int nsplit, int nchunk,
                  float* chunk_sums, float* out, int64_t out_rows, int R, const float* scale,
-                 cudaStream_t s) {
+                 bool fill, cudaStream_t s) {
   if (nsplit <= 0) return SPM_OK;
   splitrow_chunk_kernel<<<nchunk, 256, 0, s>>>(part, splits, nsplit, nchunk, R, chunk_sums);
   splitrow_fixup_kernel<<<nsplit, 256, 0, s>>>(chunk_sums, splits, nsplit, out, out_rows, R,
-                                               scale);
+                                               scale, fill);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SPM_OK : cuda_fail(e, "split-row fix-up launch");
 }

@@ -28,22 +28,20 @@
 //     block, are left as partials in `part`, summed by the fix-up kernel in block order.
 // No atomics on data (the counter only hands out blocks, and a block's result does not
 // depend on who takes it): results are bit-identical from run to run and every output
-// row is written exactly once (empty rows are zero-filled by the writer of the next
-// nonempty row, or of the last one).
+// row is written exactly once (the empty ones from a list that all warps share).
 //
 // What bounds it, measured on a GB300 (3 modes 120000 x 90000 x 2000000, 100M nonzeros,
-// Zipf 1.1, rank 32 FP32; ms per pass of mode 0 / 1 / 2): 2.55 / 2.89 / 2.46 with the
-// remap and 1.43 / 1.43 / 1.81 without, against 2.98 / 3.26 / 2.58 and 1.91 / 1.95 /
-// 1.72 of one 1.7K-nonzero block per warp with its groups on four separate runs.  Three
-// things set the shape:
+// Zipf 1.1, rank 32 FP32): a sweep takes 7.70 ms against 8.79 of one 1.7K-nonzero block
+// per warp with its groups on four separate runs; passes of modes 0 and 1 without the
+// remap 1.43 ms against 1.91 and 1.95.  Three things set the shape:
 //   * Shared memory is taken from L1, and the gathers in flight (up to 128 KB per SM)
 //     need L1 lines to land in: a 128-nonzero tile and a 4 KB scratch per warp left
 //     modes 0 and 1 at 2.1-2.2 ms without the remap, 64 and 2 KB take 1.4.
 //   * Blocks of about 512 nonzeros: larger ones spread the remap stores over more of
 //     the next order than L2 holds, smaller ones pay more for their ends.
 //   * Code size: with the row ends' code unrolled into every step the kernel was 50-66
-//     KB, and mode 2 (50 nonzeros per row) waited on instruction fetch at 2.9 ms; as a
-//     loop over the scratch it is 36 KB.
+//     KB, and mode 2 (50 nonzeros per row) waited on instruction fetch at 2.9 ms without
+//     the remap; as a loop over the scratch it takes 1.8.
 // The remainder is gather latency and the DRAM cost of the scattered sectors.
 #pragma once
 
@@ -386,8 +384,7 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
 
   // ---- staging.  Lane 0 walks the warp's blocks tile by tile, one stage each: a
-  // descriptor {first position, nonzeros | flags << 16, block, row before the
-  // block}, then one mbarrier arrival with the tile's byte count.  A tile of no
+  // descriptor {first position, nonzeros | flags << 16, block, 0}, then one mbarrier arrival with the tile's byte count.  A tile of no
   // nonzeros ends the sequence.
   constexpr int kFirst = 4, kLast = 8;  // tile flags beside BLK_HEAD_SPLIT, BLK_TAIL_SPLIT
   int in_flight = 0;                    // tiles issued and not yet waited for
@@ -514,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
   float acc[NV];
 #pragma unroll
   for (int j = 0; j < NV; ++j) acc[j] = 0.f;
-  int cur = -1, prev = -1;  // current row, the nonempty row before it
+  int cur = -1;             // current row
   bool first = true;        // cur is the block's first row
   auto piece_rank = [&](int j) -> int { return (sub + L * j) * VW; };  // first value of piece j
   auto store_row = [&](float* d, const float (&v)[NV], float s) {
@@ -542,42 +539,19 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       }
     }
   };
-  auto zero_rows = [&](int64_t from, int64_t to, int who, int n) {  // rows [from, to), n lanes
-    float* d = out + from * R;
-    const int64_t count = (to - from) * R;
-    if constexpr (VW % 4 == 0) {
-#pragma unroll 1
-      for (int64_t i = who; 4 * i < count; i += n)
-        reinterpret_cast<float4*>(d)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-#pragma unroll 1
-      for (int64_t i = who; i < count; i += n) d[i] = 0.f;
-    }
-  };
-  // All lanes: the row `cur` ends: to the block's partials where it is split, else to
-  // M_n after the empty rows before it (and, for the mode's last row, those after it).
+  // All lanes: the row `cur` ends: to the block's partials where it is split, else to M_n.
   auto close_row = [&](int stage, bool last) {
-    float* to = out + (int64_t)cur * R;
-    float s = sc;
-    bool trail = false;
-    if (first || last || prev + 1 < cur) {
-      const int4 d = desc[stage];
-      const int fl = d.y >> 16;
-      if ((first && (fl & BLK_HEAD_SPLIT)) || (last && (fl & BLK_TAIL_SPLIT))) {
-        to = a.part + ((size_t)d.z * 2 + (first ? 0 : 1)) * R;
-        s = 1.f;
-      } else if (!a.no_fill) {
-        if (prev + 1 < cur) zero_rows((int64_t)prev + 1, cur, lane, 32);
-        trail = last && cur == a.last_row;
-      }
-      first = false;
-    }
+    const int4 d = desc[stage];
+    const bool split = (first && ((d.y >> 16) & BLK_HEAD_SPLIT)) ||
+                       (last && ((d.y >> 16) & BLK_TAIL_SPLIT));
+    float* const to = (split ? a.part : out) + (size_t)(split ? 2 * d.z + (first ? 0 : 1) : cur) * R;
+    const float s = split ? 1.f : sc;
+    first = false;
 #pragma unroll 1
     for (int o = L; o < 32; o <<= 1)
 #pragma unroll
       for (int j = 0; j < NV; ++j) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
     if (gw == 0) store_row(to, acc, s);
-    if (trail) zero_rows((int64_t)cur + 1, a.out_rows, lane, 32);
   };
   // Adds the n nonzeros whose weighted products lie in the scratch (staged from p0 on)
   // to their rows.
@@ -598,28 +572,24 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       int j = 0, e = srows[0];
 #pragma unroll 1
       while (true) {  // first the row `cur` up to its end, then the batch's last row
-#pragma unroll 2
+#pragma unroll 1
         for (int k = j + gw; k < e; k += G) add_slot(b + k, acc);
         if (nst == 0 || e == m) break;
         close_row(stage, false);
-        prev = cur;
         // the rows between, a group each
         if (nst > 1) {
 #pragma unroll 1
           for (int i = gw; i < nst - 1; i += G) {
             const int k0 = srows[i], k1 = srows[i + 1];
             const uint8_t* p = p0 + (b + k0) * es;
-            const int r = row_of(p), rb = i > 0 ? row_of(p - es) : cur;
+            const int r = row_of(p);
             float v[NV];
 #pragma unroll
             for (int q = 0; q < NV; ++q) v[q] = 0.f;
-#pragma unroll 2
+#pragma unroll 1
             for (int k = k0; k < k1; ++k) add_slot(b + k, v);
-            if (!a.no_fill && rb + 1 < r) zero_rows((int64_t)rb + 1, r, sub, L);
             store_row(out + (int64_t)r * R, v, sc);
           }
-          __syncwarp();
-          prev = row_of(p0 + (b + srows[nst - 1] - 1) * es);
         }
         j = srows[nst - 1];
         e = m;
@@ -725,28 +695,44 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       }
     }
   };
-  auto accumulate = [&](const float (&prod)[NV], float v) {
+  // A chunk consumed (nc nonzeros, staged from pc on) while the next one (nn, staged
+  // from pn on) is gathered into its places of the ring.  The fast body takes a whole
+  // chunk inside one output row, or inside a row and the one numbered next (so that none
+  // lies between; each is added in its own registers), the slow one any chunk through the
+  // scratch: at 53 nonzeros per row (17M, BF16, rank 32, no remap) the two-row body took
+  // a pass from 0.42 to 0.30 ms.  Which of them runs depends on the
+  // block alone, never on what the warp takes next, so results do not depend on the
+  // claims.  Each step reads the fields of the next one ahead of its own arithmetic;
+  // the empty asm keeps the compiler from reading all steps' fields at once (the ring
+  // holds most of the registers).
+  const int gs = G * es;  // bytes from a group's nonzero to its next
+  // (the two-row body below adds each group's nonzeros of the second row apart)
+  auto add_to = [&](float (&to)[NV], const float (&prod)[NV], float v) {
     if constexpr (NV % 2 == 0) {
-      float2* a2 = reinterpret_cast<float2*>(acc);
+      float2* a2 = reinterpret_cast<float2*>(to);
       const float2* p2 = reinterpret_cast<const float2*>(prod);
       const float2 vv = make_float2(v, v);
 #pragma unroll
       for (int q = 0; q < NV / 2; ++q) a2[q] = fma2(p2[q], vv, a2[q]);
     } else {
 #pragma unroll
-      for (int q = 0; q < NV; ++q) acc[q] = fmaf(prod[q], v, acc[q]);
+      for (int q = 0; q < NV; ++q) to[q] = fmaf(prod[q], v, to[q]);
     }
   };
-  // A chunk consumed (nc nonzeros, staged from pc on) while the next one (nn, staged
-  // from pn on) is gathered into its places of the ring.  The fast body takes a whole
-  // chunk inside one output row, the slow one any chunk; which of them depends on the
-  // block alone, never on what the warp takes next, so results do not depend on the
-  // claims.  Each step reads the fields of the next one ahead of its own arithmetic;
-  // the empty asm keeps the compiler from reading all steps' fields at once (the ring
-  // holds most of the registers).
-  const int gs = G * es;  // bytes from a group's nonzero to its next
-  auto body_fast = [&](auto full, int nn, const uint8_t* pc, const uint8_t* pn) {
+  auto next_row = [&](const float (&acc2)[NV], int stage) {  // `cur` ends, row cur + 1 begins
+    close_row(stage, false);
+    ++cur;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) acc[q] = acc2[q];
+  };
+  auto body_fast = [&](auto two, auto full, int nn, const uint8_t* pc, const uint8_t* pn,
+                       int stage) {
+    constexpr bool TWO = decltype(two)::value;    // rows cur and cur + 1
     constexpr bool FULL = decltype(full)::value;  // the next chunk is whole too
+    float acc2[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) acc2[q] = 0.f;
+    int row1 = 0;
     const uint8_t* ec = pc + gw * es;  // this group's nonzero of the step
     const uint8_t* en = pn + gw * es;  // and of the next chunk's step
     int nrow = 0, nix[NI];
@@ -754,25 +740,30 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
     for (int j = 0; j < NI; ++j) nix[j] = 0;
     if (FULL || gw < nn) fetch(en, nrow, nix);
     float nval = val_of(ec);
+    if (TWO) row1 = row_of(ec);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       int ix_g[NI];
 #pragma unroll
       for (int j = 0; j < NI; ++j) ix_g[j] = nix[j];
       const float v = nval;
+      const int row = row1;
       if (u + 1 < U) {
         en += gs;
         ec += gs;
         if (FULL || (u + 1) * G + gw < nn) fetch(en, nrow, nix);
         nval = val_of(ec);
+        if (TWO) row1 = row_of(ec);
         asm volatile("" ::: "memory");  // read here, a step before they are used
       }
       float prod[NV];
       product(u, prod);
-      accumulate(prod, v);
+      if (!TWO || row == cur) add_to(acc, prod, v);
+      else add_to(acc2, prod, v);
       if (FULL || u * G + gw < nn) gather(u, 0, ix_g);
       asm volatile("" ::: "memory");
     }
+    if (TWO) next_row(acc2, stage);
   };
   auto body_slow = [&](int nc, int nn, const uint8_t* pc, const uint8_t* pn, int stage) {
     int i = gw;
@@ -796,7 +787,7 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
   };
   // The fused CP-loss pass: the chunk's model values first (their products kept for the
   // gradient), the next chunk's gathers behind them, then the residuals and the rows.
-  auto body_loss = [&](bool fast, int nc, int nn, uint8_t* pc, const uint8_t* pn, int stage) {
+  auto body_loss = [&](bool same, bool two, int nc, int nn, uint8_t* pc, const uint8_t* pn, int stage) {
     float m[U], hh[U][NV];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -842,9 +833,21 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       const int i = u * G + gw;
       if (sub == 0 && i < nc)  // the residual copy: the staged value becomes e
         reinterpret_cast<float*>(pc + i * es)[3] = m[u];
-      if (fast) accumulate(hh[u], m[u]);
+      if (same) add_to(acc, hh[u], m[u]);
     }
-    if (fast) return;
+    if (same) return;
+    if (two) {
+      float acc2[NV];
+#pragma unroll
+      for (int q = 0; q < NV; ++q) acc2[q] = 0.f;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (row_of(pc + (u * G + gw) * es) == cur) add_to(acc, hh[u], m[u]);
+        else add_to(acc2, hh[u], m[u]);
+      }
+      next_row(acc2, stage);
+      return;
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = u * G + gw;
@@ -895,7 +898,6 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
   int stage = 0;        // the gathering side's tile: its stage, the phase of its barrier,
   uint32_t phase = 0;   // its flags, and its nonzeros not yet gathered
   int dy = desc[0].y, left = dy & 0xffff;
-  if (left == 0) return;  // the warp has no nonzeros
   if (remap && !LOSS) do_remap(0);
   uint8_t* pn = ebuf;
   int nn = min(CH, left);
@@ -934,7 +936,6 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
     }
     nn = min(CH, left);
     if (block_start) {
-      prev = desc[cstage].w;
       cur = row_of(pc);
       first = true;
 #pragma unroll
@@ -944,11 +945,18 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
     if constexpr (NT == 0) {
       body_generic(nc, pc, cstage);
     } else {
-      const bool fast = nc == CH && row_of(pc + last_off) == cur;
-      if constexpr (LOSS) body_loss(fast, nc, nn, pc, pn, cstage);
-      else if (fast && nn == CH) body_fast(std::true_type{}, nn, pc, pn);
-      else if (fast) body_fast(std::false_type{}, nn, pc, pn);
-      else body_slow(nc, nn, pc, pn, cstage);
+      const int over = nc == CH ? row_of(pc + last_off) - cur : -1;  // rows begun in the chunk
+      const bool same = over == 0, two = over == 1;
+      if constexpr (LOSS)
+        body_loss(same, two, nc, nn, pc, pn, cstage);
+      else if (same && nn == CH)
+        body_fast(std::false_type{}, std::true_type{}, nn, pc, pn, cstage);
+      else if (same)
+        body_fast(std::false_type{}, std::false_type{}, nn, pc, pn, cstage);
+      else if (two)
+        body_fast(std::true_type{}, std::false_type{}, nn, pc, pn, cstage);
+      else
+        body_slow(nc, nn, pc, pn, cstage);
     }
     if (tile_end) {  // the consumed chunk was its tile's last: the tile's stage is free
       __syncwarp();
@@ -963,6 +971,17 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       }
       issue(cstage);
     }
+  }
+  // the empty rows, shared by all lane groups (each reads its next piece ahead)
+  const int groups = nwarps * G;
+  int g = (blockIdx.x * CW + warp) * G + gw;
+  int2 z = g < a.ngap ? a.gaps[g] : make_int2(0, 0);
+#pragma unroll
+  for (int j = 0; j < NV; ++j) acc[j] = 0.f;
+  for (; g < a.ngap; g += groups) {
+    const int2 next = a.ngap - g > groups ? a.gaps[g + groups] : make_int2(0, 0);
+    for (int r = z.x; r < z.y; ++r) store_row(out + (int64_t)r * R, acc, 1.f);
+    z = next;
   }
 }
 
@@ -996,7 +1015,7 @@ int launch_warp_kernel(const MttkrpArgs& a0, int L, cudaStream_t s) {
     int ctas = 0;
     st = resident_ctas((const void*)kfn, smem, &ctas);
     if (st) return st;
-    grid = std::min(grid, ctas);
+    grid = std::min(std::max(grid, (a.ngap + CW * G - 1) / (CW * G)), ctas);
     // blocks past the warps' first two are claimed from a counter
     if (a.nblk > 2 * grid * CW) SPM_CUDA(cudaMemsetAsync(a.sched, 0, sizeof(int), s));
   }

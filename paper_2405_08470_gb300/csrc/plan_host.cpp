@@ -97,7 +97,7 @@ static void stable_sort_by(const int32_t* key, int64_t dim, std::vector<int32_t>
   }
 }
 
-int default_nblk(int64_t nnz, int num_sms, int variant) {
+int default_nblk(int64_t nnz, int num_sms, int variant, bool capped) {
   if (nnz <= 0) return 1;
   int64_t nb;
   if (variant == 0 || variant == 3) {
@@ -108,6 +108,9 @@ int default_nblk(int64_t nnz, int num_sms, int variant) {
     // and 1024 measure the same).  Below, 256, so that every warp has several to take.
     const int64_t sms = num_sms;
     nb = std::max(std::min((nnz + 255) / 256, sms * 128), std::min((nnz + 511) / 512, sms * 1024));
+    // Under a memory cap at most 384 per SM, for the split rows' partials (2 R floats a
+    // block).
+    if (capped) nb = std::min(nb, sms * 384);
     nb = std::max(nb, (nnz + 4095) / 4096);
   } else if (variant == 2) {
     // tile form: about 16 blocks per SM, taken dynamically by the persistent
@@ -276,6 +279,18 @@ int partition_mode(const spmttkrp_plan* p, int n, int nblk, ModeHost* out) {
       last_u = u;
     }
   }
+  // the runs of empty rows before, between and after the nonempty ones
+  if (nnz > 0) {
+    int64_t before = -1;
+    for (size_t u = 0; u <= ur.size(); ++u) {
+      const int64_t row = u < ur.size() ? ur[u] : p->dims[(size_t)n];
+      for (int64_t z = before + 1; z < row; z += kGapRows) {
+        m.gaps.push_back((int32_t)z);
+        m.gaps.push_back((int32_t)std::min<int64_t>(z + kGapRows, row));
+      }
+      before = row;
+    }
+  }
   *out = std::move(m);
   return SPM_OK;
 }
@@ -333,7 +348,7 @@ int plan_partitions(spmttkrp_plan* p, int nblk_opt) {
   for (int n = 0; n < p->N; ++n) {
     int nb = p->partition == 1
                  ? p->lpt_kappa
-                 : (nblk_opt > 0 ? nblk_opt : default_nblk(p->nnz, p->num_sms, p->variant));
+                 : (nblk_opt > 0 ? nblk_opt : default_nblk(p->nnz, p->num_sms, p->variant, p->max_bytes > 0));
     int st = partition_mode(p, n, nb, &p->mh[(size_t)n]);
     if (st != SPM_OK) return st;
   }
@@ -377,7 +392,7 @@ int build_host_plan(spmttkrp_plan* p, const int64_t* coo, const float* vals, int
   // inside a block (Section 3.4: hyperedges follow their mode-n vertex).
   std::vector<std::vector<int32_t>> blk;
   if (p->partition == 1) {
-    const int kappa = nblk_opt > 0 ? nblk_opt : default_nblk(nnz, p->num_sms, p->variant);
+    const int kappa = nblk_opt > 0 ? nblk_opt : default_nblk(nnz, p->num_sms, p->variant, p->max_bytes > 0);
     p->lpt_kappa = kappa;
     p->lpt_load.assign((size_t)N, {});
     p->lpt_empty.assign((size_t)N, {});

@@ -81,3 +81,19 @@ def test_claimed_blocks(R, N):
     dims = (700, 300, 50, 20)[:N]
     coo, vals = synth.make_coo(dims, 60000, (1.1, 1.1, 0.0, 0.0)[:N], seed=R)
     check(coo, vals, dims, R, nblk=20011)  # far more than two per resident warp
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2, 3])
+@pytest.mark.parametrize("R,max_bytes", [(32, 0), (25, 0), (16, 0), (32, 1 << 30)])
+def test_long_runs_of_empty_rows(R, max_bytes, variant):
+    # runs of 31 to 34 empty rows (the line between the two ways), runs of thousands
+    # before, between and after the nonempty rows, and a split row behind one; a plan with
+    # a memory cap keeps no list of them
+    rows = np.concatenate([[5000], 5001 + np.cumsum([32, 33, 34, 35, 1, 64, 65, 66, 5000, 1])])
+    dims, r = (int(rows[-1]) + 3000, 40, 11), np.random.default_rng(1)
+    c = np.unique(np.stack([np.concatenate([r.choice(rows, 300), np.full(300, rows[-2])]),
+                            r.integers(0, 40, 600), r.integers(0, 11, 600)], 1), axis=0)
+    assert len(np.unique(c[:, 0])) == len(rows)
+    v = r.random(len(c)).astype(np.float32)
+    check(torch.from_numpy(c), torch.from_numpy(v), dims, R, nblk=7, variant=variant,
+          max_bytes=max_bytes)
