@@ -13,6 +13,9 @@ int launch_gram(const void* A, int dtype, int64_t I, int R, double* part, int ma
                 double* G, cudaStream_t s);
 int launch_als_prep(const double* grams, int N, int n, int R, double* work, float* vinv,
                     int* status, cudaStream_t s);
+// Blocks of the row-wise kernels (solve, scale) for I rows: one per row tile, at most nb
+// (a factor of 200 rows then leaves one partial sum per column to add, not nb).
+int als_row_blocks(int64_t I, int R, int nb);
 int launch_als_solve(const float* M, float* U, const float* vinv, int64_t I, int R,
                      double* colsq, const int* status, int nb, cudaStream_t s);
 int launch_als_lambda(const double* colsq, int nb, int R, double* lam64, float* lam_out,

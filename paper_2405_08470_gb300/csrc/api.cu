@@ -696,7 +696,9 @@ int spmttkrp_plan_query(spmttkrp_plan_t p, int what, int mode, void* dst, size_t
       o[8] = (int64_t)p->mh[(size_t)m].splits.size();
       int64_t launches = 0;
       for (int n = 0; n < N; ++n)
-        launches += 1 + (p->mh[(size_t)n].splits.empty() ? 0 : 2) +
+        launches += 1 + (p->mh[(size_t)n].splits.empty() ? 0
+                         : p->mh[(size_t)n].nchunk == (int)p->mh[(size_t)n].splits.size() ? 1
+                                                                                         : 2) +
                     (p->mh[(size_t)n].empty_rows.empty() ? 0 : 1);
       o[9] = nnz > 0 ? launches : N;
       o[10] = (int64_t)p->dev_bytes;

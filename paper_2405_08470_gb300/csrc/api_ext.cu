@@ -88,19 +88,21 @@ static int als_enqueue(spmttkrp_plan* p, void* const* factors, float* lambda,
   if ((st = launch_als_prep(p->d_gram, N, 0, R, p->d_chol, p->d_vinv, status, side))) return st;
   SPM_CUDA(cudaEventRecord(p->als_join, side));
   std::vector<const void*> cf(factors, factors + N);
+  int nb = 0;  // blocks of the mode's row kernels
   for (int n = 0; n < N; ++n) {
     const int64_t I = p->dims[(size_t)n];
+    nb = als_row_blocks(I, R, p->red_nb);
     if ((st = compute_mode(p, n, cf.data(), p->d_M, false))) return st;
     SPM_CUDA(cudaStreamWaitEvent(s, p->als_join, 0));  // V^-1 of mode n is ready
     if (!fold || R > 64) {  // the column norms (R > 64: U itself, for the scale pass)
-      if ((st = launch_als_solve(p->d_M, p->d_U, p->d_vinv, I, R, colsq, status, p->red_nb, s)))
+      if ((st = launch_als_solve(p->d_M, p->d_U, p->d_vinv, I, R, colsq, status, nb, s)))
         return st;
     }
-    if (!fold && (st = launch_als_lambda(colsq, p->red_nb, R, lam64, lambda, status, s)))
+    if (!fold && (st = launch_als_lambda(colsq, nb, R, lam64, lambda, status, s)))
       return st;
     // A_n = U / lambda, or with folding U / 1 = U itself; and <M, A_n>
     if ((st = launch_als_scale(p->d_U, p->d_M, p->d_vinv, factors[n], p->dtype,
-                               fold ? lam_one : lam64, I, R, mdot, status, p->red_nb, s)))
+                               fold ? lam_one : lam64, I, R, mdot, status, nb, s)))
       return st;
     // side: the updated factor's Gram, then the next mode's Cholesky
     SPM_CUDA(cudaEventRecord(p->als_fork, s));
@@ -114,7 +116,7 @@ static int als_enqueue(spmttkrp_plan* p, void* const* factors, float* lambda,
     SPM_CUDA(cudaEventRecord(p->als_join, side));
   }
   SPM_CUDA(cudaStreamWaitEvent(s, p->als_join, 0));
-  return launch_als_fit(p->d_gram, N, R, fold ? lam_one : lam64, mdot, p->red_nb, p->normx2, fit,
+  return launch_als_fit(p->d_gram, N, R, fold ? lam_one : lam64, mdot, nb, p->normx2, fit,
                         status, s);
 }
 

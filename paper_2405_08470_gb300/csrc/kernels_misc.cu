@@ -96,10 +96,24 @@ int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s) {
 // per split row adds its chunk sums in chunk order, writes the row once and (fill)
 // zeroes the empty rows before it (and after it, for the last nonempty row).  A
 // row spread over thousands of blocks (a Zipf head row) is summed by many CTAs.
+// Where no split row has more than one chunk (small tensors, where the launches are what
+// takes the time) pass 1 writes the rows themselves (direct) and pass 2 is not launched.
+__device__ void zero_gaps(const SplitRow& sr, float* __restrict__ out, int64_t out_rows, int R) {
+  const int64_t gap0 = (int64_t)sr.prev_row + 1, ngap = ((int64_t)sr.row - gap0) * R;
+  for (int64_t i = threadIdx.x; i < ngap; i += blockDim.x) out[gap0 * R + i] = 0.f;
+  if (sr.is_last) {
+    const int64_t t0 = (int64_t)sr.row + 1, nt = (out_rows - t0) * R;
+    for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) out[t0 * R + i] = 0.f;
+  }
+}
+
 __global__ void __launch_bounds__(256) splitrow_chunk_kernel(const float* __restrict__ part,
                                                              const SplitRow* __restrict__ splits,
                                                              int nsplit, int nchunk, int R,
-                                                             float* __restrict__ chunk_sums) {
+                                                             float* __restrict__ chunk_sums,
+                                                             float* __restrict__ out,
+                                                             int64_t out_rows, const float* scale,
+                                                             bool fill, bool direct) {
   __shared__ float red[8][kMaxRank];
   const int c = blockIdx.x;
   if (c >= nchunk) return;
@@ -127,8 +141,10 @@ __global__ void __launch_bounds__(256) splitrow_chunk_kernel(const float* __rest
     float acc = 0.f;
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc += red[q][r];
-    chunk_sums[(size_t)c * R + r] = acc;
+    if (direct) out[(int64_t)sr.row * R + r] = acc * (scale ? __ldg(scale) : 1.0f);
+    else chunk_sums[(size_t)c * R + r] = acc;
   }
+  if (direct && fill) zero_gaps(sr, out, out_rows, R);
 }
 
 __global__ void __launch_bounds__(256) splitrow_fixup_kernel(const float* __restrict__ chunk_sums,
@@ -140,13 +156,7 @@ __global__ void __launch_bounds__(256) splitrow_fixup_kernel(const float* __rest
   const SplitRow sr = splits[blockIdx.x];
   const float sc = scale ? __ldg(scale) : 1.0f;
   const int nc = (sr.last_blk - sr.first_blk + kFixChunk) / kFixChunk;
-  const int64_t gap0 = (int64_t)sr.prev_row + 1, ngap = ((int64_t)sr.row - gap0) * R;
-  if (fill)  // (forms 0 and 3 zero the empty rows from their list)
-    for (int64_t i = threadIdx.x; i < ngap; i += blockDim.x) out[gap0 * R + i] = 0.f;
-  if (fill && sr.is_last) {
-    const int64_t t0 = (int64_t)sr.row + 1, nt = (out_rows - t0) * R;
-    for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) out[t0 * R + i] = 0.f;
-  }
+  if (fill) zero_gaps(sr, out, out_rows, R);  // (forms 0 and 3 zero them from their list)
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
     float acc = 0.f;
     for (int q = 0; q < nc; ++q) acc += chunk_sums[(size_t)(sr.chunk0 + q) * R + r];
@@ -158,9 +168,12 @@ int launch_fixup(const float* part, const SplitRow* splits, int nsplit, int nchu
                  float* chunk_sums, float* out, int64_t out_rows, int R, const float* scale,
                  bool fill, cudaStream_t s) {
   if (nsplit <= 0) return SPM_OK;
-  splitrow_chunk_kernel<<<nchunk, 256, 0, s>>>(part, splits, nsplit, nchunk, R, chunk_sums);
-  splitrow_fixup_kernel<<<nsplit, 256, 0, s>>>(chunk_sums, splits, nsplit, out, out_rows, R,
-                                               scale, fill);
+  const bool direct = nchunk == nsplit;
+  splitrow_chunk_kernel<<<nchunk, 256, 0, s>>>(part, splits, nsplit, nchunk, R, chunk_sums, out,
+                                               out_rows, scale, fill, direct);
+  if (!direct)
+    splitrow_fixup_kernel<<<nsplit, 256, 0, s>>>(chunk_sums, splits, nsplit, out, out_rows, R,
+                                                 scale, fill);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SPM_OK : cuda_fail(e, "split-row fix-up launch");
 }
