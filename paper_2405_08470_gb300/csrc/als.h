@@ -22,9 +22,11 @@ int launch_als_lambda(const double* colsq, int nb, int R, double* lam64, float* 
                       const int* status, cudaStream_t s);
 // R <= 64: U is not read (nor written by launch_als_solve, which then leaves the
 // column norms only); the scale pass forms M V^-1 again from M and vinv.
+// nc > 0 (R <= 64): lambda is formed here from the nc partial column sums in colsq
+// (launch_als_solve's) and written to lam64 and lam_out.
 int launch_als_scale(const float* U, const float* M, const float* vinv, void* A, int dtype,
-                     const double* lam64, int64_t I, int R, double* mdot, const int* status,
-                     int nb, cudaStream_t s);
+                     double* lam64, int64_t I, int R, double* mdot, const int* status,
+                     int nb, const double* colsq, int nc, float* lam_out, cudaStream_t s);
 int launch_fill_f64(double* p, int n, double v, cudaStream_t s);
 // The end of a column-scale-folded loop: lambda_r = prod_k sqrt(G_k[r, r]) and
 // every factor divided by its column norms (the Grams must be the stored factors').

@@ -72,7 +72,7 @@ static int als_enqueue(spmttkrp_plan* p, void* const* factors, float* lambda,
   int* status = reinterpret_cast<int*>(p->d_scal);
   double* fit = p->d_scal + 1;
   double* lam64 = p->d_scal + 8;
-  const double* lam_one = p->d_scal + 8 + R;
+  double* lam_one = p->d_scal + 8 + R;
   double* colsq = p->d_red;
   double* mdot = p->d_red + (size_t)p->red_nb * R;
   cudaStream_t s = p->stream, side = p->als_side;
@@ -98,11 +98,14 @@ static int als_enqueue(spmttkrp_plan* p, void* const* factors, float* lambda,
       if ((st = launch_als_solve(p->d_M, p->d_U, p->d_vinv, I, R, colsq, status, nb, s)))
         return st;
     }
-    if (!fold && (st = launch_als_lambda(colsq, nb, R, lam64, lambda, status, s)))
+    // few partials: the scale pass forms lambda itself
+    const int nc = !fold && R <= 64 && nb <= 8 ? nb : 0;
+    if (!fold && nc == 0 && (st = launch_als_lambda(colsq, nb, R, lam64, lambda, status, s)))
       return st;
     // A_n = U / lambda, or with folding U / 1 = U itself; and <M, A_n>
     if ((st = launch_als_scale(p->d_U, p->d_M, p->d_vinv, factors[n], p->dtype,
-                               fold ? lam_one : lam64, I, R, mdot, status, nb, s)))
+                               fold ? lam_one : lam64, I, R, mdot, status, nb, colsq, nc, lambda,
+                               s)))
       return st;
     // side: the updated factor's Gram, then the next mode's Cholesky
     SPM_CUDA(cudaEventRecord(p->als_fork, s));

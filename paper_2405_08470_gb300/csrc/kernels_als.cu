@@ -411,10 +411,12 @@ template <typename T, int RP, bool SCALE>
 __global__ void __launch_bounds__(256) als_rows_kernel(const float* __restrict__ M,
                                                        const float* __restrict__ vinv,
                                                        T* __restrict__ A,
-                                                       const double* __restrict__ lam64,
+                                                       double* __restrict__ lam64,
                                                        int64_t I, int R,
                                                        double* __restrict__ part,
-                                                       const int* __restrict__ status) {
+                                                       const int* __restrict__ status,
+                                                       const double* __restrict__ colsq, int nc,
+                                                       float* __restrict__ lam_out) {
   constexpr int CB = RP / 4, RS = 256 / CB, RT = 4 * RS, LD = RP + 1;
   __shared__ float Ms[RT * LD];
   __shared__ __align__(16) float Vs[RP * RP];
@@ -425,10 +427,27 @@ __global__ void __launch_bounds__(256) als_rows_kernel(const float* __restrict__
     const int j = e / RP, c = e % RP;
     Vs[e] = (j < R && c < R) ? vinv[j * R + c] : 0.f;
   }
+  __shared__ float invs[RP];  // SCALE: 1 / lambda
+  if (SCALE && tid < RP) {
+    double l = 1.0;
+    if (tid < R && nc > 0) {  // few partials: every block adds them itself (one launch less)
+      double s = 0.0;
+      for (int q = 0; q < nc; ++q) s += colsq[(size_t)q * R + tid];
+      l = sqrt(s);
+      if (blockIdx.x == 0) {
+        lam64[tid] = l;
+        lam_out[tid] = (float)l;
+      }
+    } else if (tid < R) {
+      l = lam64[tid];
+    }
+    invs[tid] = tid < R ? (float)(1.0 / l) : 0.f;
+  }
+  __syncthreads();
   float inv[4], sum[4];
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
-    inv[b] = (SCALE && c0 + b < R) ? (float)(1.0 / lam64[c0 + b]) : 0.f;
+    inv[b] = SCALE ? invs[c0 + b] : 0.f;
     sum[b] = 0.f;
   }
   const int64_t ntiles = (I + RT - 1) / RT;
@@ -480,10 +499,21 @@ __global__ void __launch_bounds__(256) als_rows_kernel(const float* __restrict__
 #pragma unroll
   for (int b = 0; b < 4; ++b) red[rs][c0 + b] = sum[b];
   __syncthreads();
-  for (int c = tid; c < R; c += 256) {
+  // column c: 256 / RP threads add RS / (256 / RP) entries each, then one adds theirs
+  constexpr int TP = 256 / RP, EP = RS / TP;
+  __shared__ double red2[TP][RP];
+  {
     double acc = 0.0;
-    for (int q = 0; q < RS; ++q) acc += (double)red[q][c];
-    part[(size_t)blockIdx.x * R + c] = acc;
+#pragma unroll
+    for (int q = 0; q < EP; ++q) acc += (double)red[(tid / RP) * EP + q][tid % RP];
+    red2[tid / RP][tid % RP] = acc;
+  }
+  __syncthreads();
+  if (tid < R) {
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < TP; ++q) acc += red2[q][tid];
+    part[(size_t)blockIdx.x * R + tid] = acc;
   }
 }
 
@@ -725,13 +755,13 @@ int launch_als_solve(const float* M, float* U, const float* vinv, int64_t I, int
   const int cc = (R + 31) / 32;
   if (R <= 16)  // column norms only: the scale pass forms U again
     als_rows_kernel<float, 16, false><<<nb, 256, 0, s>>>(M, vinv, nullptr, nullptr, I, R, colsq,
-                                                          status);
+                                                          status, nullptr, 0, nullptr);
   else if (R <= 32)
     als_rows_kernel<float, 32, false><<<nb, 256, 0, s>>>(M, vinv, nullptr, nullptr, I, R, colsq,
-                                                          status);
+                                                          status, nullptr, 0, nullptr);
   else if (R <= 64)
     als_rows_kernel<float, 64, false><<<nb, 256, 0, s>>>(M, vinv, nullptr, nullptr, I, R, colsq,
-                                                          status);
+                                                          status, nullptr, 0, nullptr);
   else if (cc <= 1) solve_cc<1>(M, U, vinv, I, R, colsq, status, nb, s);
   else if (cc <= 2) solve_cc<2>(M, U, vinv, I, R, colsq, status, nb, s);
   else if (cc <= 4) solve_cc<4>(M, U, vinv, I, R, colsq, status, nb, s);
@@ -755,26 +785,30 @@ static void scale_cc(const float* U, const float* M, void* A, const double* lam6
 }
 
 template <typename T>
-static void rows_scale(const float* M, const float* vinv, void* A, const double* lam64, int64_t I,
-                       int R, double* mdot, const int* status, int nb, cudaStream_t s) {
+static void rows_scale(const float* M, const float* vinv, void* A, double* lam64, int64_t I,
+                       int R, double* mdot, const int* status, int nb, const double* colsq, int nc,
+                       float* lam_out, cudaStream_t s) {
   T* At = static_cast<T*>(A);
   if (R <= 16)
-    als_rows_kernel<T, 16, true><<<nb, 256, 0, s>>>(M, vinv, At, lam64, I, R, mdot, status);
+    als_rows_kernel<T, 16, true><<<nb, 256, 0, s>>>(M, vinv, At, lam64, I, R, mdot, status, colsq,
+                                                    nc, lam_out);
   else if (R <= 32)
-    als_rows_kernel<T, 32, true><<<nb, 256, 0, s>>>(M, vinv, At, lam64, I, R, mdot, status);
+    als_rows_kernel<T, 32, true><<<nb, 256, 0, s>>>(M, vinv, At, lam64, I, R, mdot, status, colsq,
+                                                    nc, lam_out);
   else
-    als_rows_kernel<T, 64, true><<<nb, 256, 0, s>>>(M, vinv, At, lam64, I, R, mdot, status);
+    als_rows_kernel<T, 64, true><<<nb, 256, 0, s>>>(M, vinv, At, lam64, I, R, mdot, status, colsq,
+                                                    nc, lam_out);
 }
 
 int launch_als_scale(const float* U, const float* M, const float* vinv, void* A, int dtype,
-                     const double* lam64, int64_t I, int R, double* mdot, const int* status,
-                     int nb, cudaStream_t s) {
+                     double* lam64, int64_t I, int R, double* mdot, const int* status,
+                     int nb, const double* colsq, int nc, float* lam_out, cudaStream_t s) {
   const int cc = (R + 31) / 32;
   if (R <= 64) {
     if (dtype == SPM_DTYPE_BF16)
-      rows_scale<__nv_bfloat16>(M, vinv, A, lam64, I, R, mdot, status, nb, s);
+      rows_scale<__nv_bfloat16>(M, vinv, A, lam64, I, R, mdot, status, nb, colsq, nc, lam_out, s);
     else
-      rows_scale<float>(M, vinv, A, lam64, I, R, mdot, status, nb, s);
+      rows_scale<float>(M, vinv, A, lam64, I, R, mdot, status, nb, colsq, nc, lam_out, s);
   } else if (dtype == SPM_DTYPE_BF16) {
     if (cc <= 1) scale_cc<__nv_bfloat16, 1>(U, M, A, lam64, I, R, mdot, status, nb, s);
     else if (cc <= 2) scale_cc<__nv_bfloat16, 2>(U, M, A, lam64, I, R, mdot, status, nb, s);

@@ -105,9 +105,14 @@ int default_nblk(int64_t nnz, int num_sms, int variant, bool capped) {
     // nonzeros on they hold 512 (the remap's stores then stay within what L2 holds: a
     // 30M-nonzero sweep takes 2.28 ms with 512 and 2.37 with 1024; 256 pay more for
     // their ends, 2.30), up to 1024 blocks per SM (larger blocks beyond: at 100M, 640
-    // and 1024 measure the same).  Below, 256, so that every warp has several to take.
+    // and 1024 measure the same).  Below, 256, so that every warp has several to take,
+    // and on tensors too small for that fewer, down to 64, so that every SM has some (a
+    // sweep of 50K nonzeros takes 35 us with 64 and 47 with 256; of 200K, 52 with 192 and
+    // 60 with 256).
     const int64_t sms = num_sms;
-    nb = std::max(std::min((nnz + 255) / 256, sms * 128), std::min((nnz + 511) / 512, sms * 1024));
+    const int64_t few = std::min<int64_t>(256, std::max<int64_t>(64, nnz / (sms * 8)));
+    nb = std::max(std::min((nnz + few - 1) / few, sms * 128),
+                  std::min((nnz + 511) / 512, sms * 1024));
     // Under a memory cap at most 384 per SM, for the split rows' partials (2 R floats a
     // block).
     if (capped) nb = std::min(nb, sms * 384);
