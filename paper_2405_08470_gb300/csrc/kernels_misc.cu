@@ -93,7 +93,7 @@ int launch_mttkrp(const MttkrpArgs& a, cudaStream_t s) {
 // bit-identical run to run).  Pass 1: one CTA per chunk of up to kFixChunk
 // consecutive blocks of a split row; warp w sums the chunk's blocks w, w+8, ...
 // (lanes over R) and the 8 warp sums are added in warp order.  Pass 2: one CTA
-// per split row adds its chunk sums in chunk order, writes the row once and (fill)
+// per split row adds its chunk sums the same way, writes the row once and (fill)
 // zeroes the empty rows before it (and after it, for the last nonempty row).  A
 // row spread over thousands of blocks (a Zipf head row) is summed by many CTAs.
 // Where no split row has more than one chunk (small tensors, where the launches are what
@@ -152,14 +152,25 @@ __global__ void __launch_bounds__(256) splitrow_fixup_kernel(const float* __rest
                                                              int nsplit, float* __restrict__ out,
                                                              int64_t out_rows, int R,
                                                              const float* scale, bool fill) {
+  __shared__ float red[8][kMaxRank];
   if ((int)blockIdx.x >= nsplit) return;
   const SplitRow sr = splits[blockIdx.x];
   const float sc = scale ? __ldg(scale) : 1.0f;
   const int nc = (sr.last_blk - sr.first_blk + kFixChunk) / kFixChunk;
   if (fill) zero_gaps(sr, out, out_rows, R);  // (forms 0 and 3 zero them from their list)
+  // warp w adds chunks w, w + 8, ..; a row of a hundred chunks is then neither a chain of
+  // a hundred loads nor one of a hundred roundings
+  const int w = threadIdx.x >> 5;
+  for (int r = threadIdx.x & 31; r < R; r += 32) {
+    float acc = 0.f;
+    for (int q = w; q < nc; q += 8) acc += chunk_sums[(size_t)(sr.chunk0 + q) * R + r];
+    red[w][r] = acc;
+  }
+  __syncthreads();
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
     float acc = 0.f;
-    for (int q = 0; q < nc; ++q) acc += chunk_sums[(size_t)(sr.chunk0 + q) * R + r];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc += red[q][r];
     out[(int64_t)sr.row * R + r] = acc * sc;
   }
 }
