@@ -92,8 +92,8 @@ int launch_mttkrp_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
   switch (c.RC) {
     case 1: return launch_warp_kernel<0, float, 1, 1, 4>(a, c.L, s);
     case 2: return launch_warp_kernel<0, float, 1, 2, 4>(a, c.L, s);
-    case 4: return launch_warp_kernel<0, float, 1, 4, 2>(a, c.L, s);
-    default: return launch_warp_kernel<0, float, 1, 8, 1>(a, c.L, s);
+    case 4: return launch_warp_kernel<0, float, 1, 4, 4>(a, c.L, s);
+    default: return launch_warp_kernel<0, float, 1, 8, 2>(a, c.L, s);
   }
 }
 

@@ -73,15 +73,11 @@ inline LaneCfg warp_lane_config(int R, int dtype, size_t factor_align, size_t ou
 // ------------------------------------------------------------ stored nonzeros
 
 // Index k of a stored nonzeros (plain: word k; packed: its bit field).
+// A field of at most 31 bits lies in two neighbouring words: one funnel shift.
 __device__ __forceinline__ uint32_t pk_field(const uint32_t* w, int off, int b) {
-  uint64_t x;
-  if (off < 32)
-    x = (((uint64_t)w[1] << 32) | w[0]) >> off;
-  else if (off < 64)
-    x = (((uint64_t)w[2] << 32) | w[1]) >> (off - 32);
-  else
-    x = (uint64_t)(w[2] >> (off - 64));
-  return (uint32_t)x & ((1u << b) - 1u);
+  const uint32_t lo = off < 32 ? w[0] : (off < 64 ? w[1] : w[2]);
+  const uint32_t hi = off < 32 ? w[1] : (off < 64 ? w[2] : 0u);
+  return __funnelshift_r(lo, hi, off & 31) & ((1u << b) - 1u);
 }
 __device__ __forceinline__ int elem_index(const uint8_t* ep, int k, const PackInfo& pk) {
   const uint32_t* w = reinterpret_cast<const uint32_t*>(ep);

@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
   };
   // Runtime number of modes: a chunk's nonzeros are gathered mode by mode when it is
   // consumed, each slice multiplied in as it lands.
-  auto body_generic = [&](int nc, const uint8_t* pc, int stage) {
+  auto body_generic = [&](bool same, int nc, const uint8_t* pc, int stage) {
     float pr[U][NV];
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -882,6 +882,11 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
           for (int c = 0; c < VW; ++c) pr[u][j * VW + c] *= x[c];
         }
       }
+    }
+    if (same) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) add_to(acc, pr[u], val_of(pc + (u * G + gw) * es));
+      return;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -943,7 +948,7 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       block_start = false;
     }
     if constexpr (NT == 0) {
-      body_generic(nc, pc, cstage);
+      body_generic(nc == CH && row_of(pc + last_off) == cur, nc, pc, cstage);
     } else {
       const int over = nc == CH ? row_of(pc + last_off) - cur : -1;  // rows begun in the chunk
       const bool same = over == 0, two = over == 1;
