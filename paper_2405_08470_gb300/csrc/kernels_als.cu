@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(256) als_sweep_kernel(const double* __restrict
                                                         int* __restrict__ status) {
   constexpr int T = 256 / RP, Q = RP / T;  // threads per row, columns per thread
   __shared__ double colp[2][RP];  // the pivot's column, double-buffered
-  __shared__ double rdiag[2];     // 1 / pivot
+  __shared__ double rdiag[2];     // 1 / pivot (0: not positive or not finite)
   __shared__ int bad;
   const int tid = threadIdx.x, i = tid / T, g = tid % T;
   if (tid == 0) bad = *status;
@@ -215,17 +215,17 @@ __global__ void __launch_bounds__(256) als_sweep_kernel(const double* __restrict
     for (int q = 0; q < Q; ++q)
       if (g + T * q == p && i < R) {
         colp[p & 1][i] = v[q];
-        if (i == p) {
-          if (!(v[q] > 0.0) || !isfinite(v[q])) bad = 1;
-          rdiag[p & 1] = 1.0 / v[q];
-        }
+        if (i == p) rdiag[p & 1] = v[q] > 0.0 && isfinite(v[q]) ? 1.0 / v[q] : 0.0;
       }
   };
   publish(0);
   __syncthreads();
   for (int p = 0; p < R; ++p) {
-    if (bad) break;
     const double rd = rdiag[p & 1];
+    if (!(rd > 0.0)) {  // not SPD: every thread reads the same value here
+      if (tid == 0) *status = SPM_ERR_NOT_SPD;
+      return;
+    }
     const double ci = i < R ? colp[p & 1][i] : 0.0, si = ci * rd;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
@@ -237,10 +237,6 @@ __global__ void __launch_bounds__(256) als_sweep_kernel(const double* __restrict
     }
     if (p + 1 < R) publish(p + 1);
     __syncthreads();
-  }
-  if (bad) {
-    if (tid == 0) *status = SPM_ERR_NOT_SPD;
-    return;
   }
 #pragma unroll
   for (int q = 0; q < Q; ++q)
