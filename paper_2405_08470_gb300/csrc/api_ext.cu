@@ -129,8 +129,13 @@ static void drop_graphs(std::vector<GraphCache>& v) {
   v.clear();
 }
 
-// Re-cuts every mode into nblk blocks and switches the kernel form / tile / ring.
+// Re-cuts every mode into nblk blocks and switches the kernel form / tile / ring.  Every
+// captured graph (sweeps, ALS iterations, ALS loops) holds the addresses of the block
+// tables and partials, so all of them go before the tables do.
 static int apply_config(spmttkrp_plan* p, int nblk, int tile, int variant, int stages) {
+  drop_graphs(p->sweep_graphs);
+  drop_graphs(p->als_graphs);
+  drop_graphs(p->als_run_graphs);
   for (int n = 0; n < p->N; ++n) {
     int st = partition_mode(p, n, nblk, &p->mh[(size_t)n]);
     if (st) return st;
@@ -140,8 +145,6 @@ static int apply_config(spmttkrp_plan* p, int nblk, int tile, int variant, int s
   p->tile = tile;
   p->variant = variant;
   p->stages = stages;
-  drop_graphs(p->sweep_graphs);
-  drop_graphs(p->als_graphs);
   return SPM_OK;
 }
 
