@@ -60,84 +60,60 @@ static void dfree(void* ptr) {
   if (ptr) cudaFree(ptr);
 }
 
-// Uploads one mode's block descriptors and split table (after (re)partitioning).
+// Uploads one mode's block descriptors, split table and lists of empty rows (after
+// (re)partitioning).  The old tables go first, so that a re-cut needs no more memory than
+// the larger of the two; a count is set only once its table is there, and `ready` last: a
+// pass over a mode whose upload ran out of memory is refused (run_mode), never launched
+// on a table that is missing.
 int upload_mode_tables(spmttkrp_plan* p, int n) {
   ModeHost& h = p->mh[(size_t)n];
   ModeDev& d = p->md[(size_t)n];
-  if (d.blkinfo) {
-    cudaFree(d.blkinfo);
-    p->dev_bytes -= std::max<size_t>((size_t)d.nblk * sizeof(int4), 16);
-    d.blkinfo = nullptr;
-  }
-  if (d.splits) {
-    cudaFree(d.splits);
-    p->dev_bytes -= std::max<size_t>((size_t)d.nsplit * sizeof(SplitRow), 16);
-    d.splits = nullptr;
-  }
-  if (d.empty_rows) {
-    cudaFree(d.empty_rows);
-    p->dev_bytes -= std::max<size_t>((size_t)d.nempty * sizeof(int32_t), 16);
-    d.empty_rows = nullptr;
-  }
-  if (d.gaps) {
-    cudaFree(d.gaps);
-    p->dev_bytes -= std::max<size_t>((size_t)d.ngap * sizeof(int2), 16);
-    d.gaps = nullptr;
-  }
-  d.nblk = h.nblk;
-  d.nsplit = (int)h.splits.size();
-  d.nchunk = h.nchunk;
+  auto drop = [&](auto*& ptr, size_t bytes) {
+    if (!ptr) return;
+    cudaFree(ptr);
+    p->dev_bytes -= std::max<size_t>(bytes, 16);
+    ptr = nullptr;
+  };
+  d.ready = false;
+  drop(d.blkinfo, (size_t)d.nblk * sizeof(int4));
+  drop(d.splits, (size_t)d.nsplit * sizeof(SplitRow));
+  drop(d.empty_rows, (size_t)d.nempty * sizeof(int32_t));
+  drop(d.gaps, (size_t)d.ngap * sizeof(int2));
+  d.nblk = d.nsplit = d.nchunk = d.nempty = d.ngap = 0;
   d.last_row = h.last_row;
-  int st = plan_dalloc(p, (void**)&d.blkinfo, (size_t)d.nblk * sizeof(int4));
+  d.has_gaps = !h.gaps.empty();
+  // table <- `count` entries of `src`, then the count
+  auto table = [&](auto*& ptr, int& have, const void* src, size_t count) -> int {
+    const size_t bytes = count * sizeof(*ptr);
+    int st = plan_dalloc(p, (void**)&ptr, bytes);
+    if (st) return st;
+    have = (int)count;
+    if (bytes) SPM_CUDA(cudaMemcpyAsync(ptr, src, bytes, cudaMemcpyHostToDevice, p->stream));
+    return SPM_OK;
+  };
+  int st = table(d.blkinfo, d.nblk, h.blkinfo.data(), (size_t)h.nblk);
+  if (!st) st = table(d.splits, d.nsplit, h.splits.data(), h.splits.size());
+  if (!st && !h.empty_rows.empty())
+    st = table(d.empty_rows, d.nempty, h.empty_rows.data(), h.empty_rows.size());
+  // (under a memory cap no list of empty rows: the output is zeroed first)
+  if (!st && d.has_gaps && !p->max_bytes)
+    st = table(d.gaps, d.ngap, h.gaps.data(), h.gaps.size() / 2);
   if (st) return st;
-  st = plan_dalloc(p, (void**)&d.splits, (size_t)d.nsplit * sizeof(SplitRow));
-  if (st) return st;
-  SPM_CUDA(cudaMemcpyAsync(d.blkinfo, h.blkinfo.data(), (size_t)d.nblk * sizeof(int4),
-                           cudaMemcpyHostToDevice, p->stream));
-  if (d.nsplit)
-    SPM_CUDA(cudaMemcpyAsync(d.splits, h.splits.data(), (size_t)d.nsplit * sizeof(SplitRow),
-                             cudaMemcpyHostToDevice, p->stream));
-  d.nempty = (int)h.empty_rows.size();
-  if (d.nempty) {
-    st = plan_dalloc(p, (void**)&d.empty_rows, (size_t)d.nempty * sizeof(int32_t));
-    if (st) return st;
-    SPM_CUDA(cudaMemcpyAsync(d.empty_rows, h.empty_rows.data(), (size_t)d.nempty * sizeof(int32_t),
-                             cudaMemcpyHostToDevice, p->stream));
-  }
-  d.ngap = (int)(h.gaps.size() / 2);
-  d.has_gaps = d.ngap > 0;
-  if (p->max_bytes) d.ngap = 0;  // under a memory cap no list: the output is zeroed first
-  if (d.ngap) {
-    st = plan_dalloc(p, (void**)&d.gaps, (size_t)d.ngap * sizeof(int2));
-    if (st) return st;
-    SPM_CUDA(cudaMemcpyAsync(d.gaps, h.gaps.data(), (size_t)d.ngap * sizeof(int2),
-                             cudaMemcpyHostToDevice, p->stream));
-  }
-  // fix-up scratch: one R-float sum per chunk of a split row's blocks
-  const size_t fneed = (size_t)std::max(d.nchunk, 1) * p->R;
-  if (fneed > p->fixsum_cap) {
-    if (p->d_fixsum) {
-      cudaFree(p->d_fixsum);
-      p->dev_bytes -= std::max<size_t>(p->fixsum_cap * 4, 16);
-      p->d_fixsum = nullptr;
-    }
-    st = plan_dalloc(p, (void**)&p->d_fixsum, fneed * 4);
-    if (st) return st;
-    p->fixsum_cap = fneed;
-  }
-  // partial-sum buffer: 2 slots of R floats per block
-  size_t need = (size_t)d.nblk * 2 * p->R;
-  if (need > p->part_cap) {
-    if (p->d_part) {
-      cudaFree(p->d_part);
-      p->dev_bytes -= std::max<size_t>(p->part_cap * 4, 16);
-      p->d_part = nullptr;
-    }
-    st = plan_dalloc(p, (void**)&p->d_part, need * 4);
-    if (st) return st;
-    p->part_cap = need;
-  }
+  d.nchunk = h.nchunk;
+  // fix-up scratch: one R-float sum per chunk of a split row's blocks; and the partials: 2
+  // slots of R floats per block
+  auto grow = [&](float*& ptr, size_t& cap, size_t need) -> int {
+    if (need <= cap) return SPM_OK;
+    drop(ptr, cap * 4);
+    cap = 0;
+    int e = plan_dalloc(p, (void**)&ptr, need * 4);
+    if (e == SPM_OK) cap = need;
+    return e;
+  };
+  if ((st = grow(p->d_fixsum, p->fixsum_cap, (size_t)std::max(d.nchunk, 1) * p->R))) return st;
+  if ((st = grow(p->d_part, p->part_cap, (size_t)d.nblk * 2 * p->R))) return st;
   SPM_CUDA(cudaStreamSynchronize(p->stream));  // host vectors may change after return
+  d.ready = true;
   return SPM_OK;
 }
 
@@ -224,6 +200,9 @@ int run_mode(spmttkrp_plan* p, int mode, const void* const* factors, float* out,
              const uint8_t* ein, uint8_t* eout, const float* scale, double* loss_part) {
   if (p->nnz == 0) return launch_zero_rows(out, p->dims[(size_t)mode], p->R, p->stream);
   const ModeDev& d = p->md[(size_t)mode];
+  if (!d.ready || p->part_cap < (size_t)d.nblk * 2 * p->R ||
+      p->fixsum_cap < (size_t)std::max(d.nchunk, 1) * p->R)
+    return fail(SPM_ERR_STATE, "the plan's block tables could not be allocated");
   MttkrpArgs a;
   std::memset(&a, 0, sizeof(a));
   a.elems_in = ein;

@@ -136,11 +136,20 @@ static int apply_config(spmttkrp_plan* p, int nblk, int tile, int variant, int s
   drop_graphs(p->sweep_graphs);
   drop_graphs(p->als_graphs);
   drop_graphs(p->als_run_graphs);
+  std::vector<int> before;
+  for (const ModeHost& h : p->mh) before.push_back(h.nblk);
+  auto recut = [&](int n, int nb) {
+    int st = partition_mode(p, n, nb, &p->mh[(size_t)n]);
+    return st ? st : upload_mode_tables(p, n);
+  };
   for (int n = 0; n < p->N; ++n) {
-    int st = partition_mode(p, n, nblk, &p->mh[(size_t)n]);
-    if (st) return st;
-    st = upload_mode_tables(p, n);
-    if (st) return st;
+    const int st = recut(n, nblk);
+    if (st == SPM_OK) continue;
+    // the new tables do not fit: back to the blocks that did (a mode that cannot even have
+    // those stays without tables, and its passes are refused)
+    const std::string why = spmttkrp_last_error();
+    for (int m = 0; m < p->N; ++m) (void)recut(m, before[(size_t)m]);
+    return fail(st, why);
   }
   p->tile = tile;
   p->variant = variant;
@@ -442,6 +451,7 @@ int cp_loss_fwd_ex(spmttkrp_plan_t p, const void* const* factors, float* loss, i
         cudaFree(p->d_lpart);
         p->dev_bytes -= std::max<size_t>(p->lpart_cap * 8, 16);
         p->d_lpart = nullptr;
+        p->lpart_cap = 0;
       }
       if ((st = plan_dalloc(p, (void**)&p->d_lpart, need * 8))) return st;
       p->lpart_cap = need;

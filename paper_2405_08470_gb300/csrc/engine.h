@@ -70,6 +70,7 @@ struct ModeHost {
 
 // Device tables of one mode.
 struct ModeDev {
+  bool ready = false;  // all tables below are on the device (upload_mode_tables)
   int nblk = 0;
   int nsplit = 0;
   int last_row = -1;

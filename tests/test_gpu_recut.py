@@ -6,7 +6,7 @@ import torch
 
 import oracle as O
 import synth
-from paper_2405_08470_gb300 import Plan
+from paper_2405_08470_gb300 import Plan, SpmError
 
 pytestmark = pytest.mark.gpu
 
@@ -36,4 +36,37 @@ def test_als_loop_after_a_recut_uses_the_new_tables():
     assert O.relerr(lam.cpu().numpy(), lo) <= 1e-5
     for k in range(3):
         assert O.relerr(F[k].cpu().numpy(), Fo[k]) <= 1e-5, k
+    p.close()
+
+
+@pytest.mark.parametrize("dims,skew", [((300, 200, 100), (1.1, 1.1, 0.0)),
+                                       ((3000, 40, 20, 10), (0.0, 1.1, 0.0, 0.0))])
+def test_recut_that_does_not_fit_leaves_the_plan_as_it_was(dims, skew):
+    """A plan at its memory cap: the autotuner's larger block counts need larger tables and
+    partials than the cap allows, which is a status; the plan keeps the blocks it had and
+    computes with them (FP32 bar of the other parity tests)."""
+    R, N = 32, len(dims)
+    coo, vals = synth.make_coo(dims, 20_000, skew, seed=N)
+    c, v = coo.numpy(), vals.numpy()
+    probe = Plan(c, v, dims, R, max_bytes=1 << 30)
+    need = probe.info()["device_bytes"]
+    probe.close()
+    p = Plan(c, v, dims, R, max_bytes=need + (64 << 10))
+    before = [p.info(n)["nblk"] for n in range(N)]
+    F = [f.cuda() for f in synth.make_factors(dims, R, seed=7)]
+    outs = [torch.empty(d, R, device="cuda") for d in dims]
+    p.sweep(F, outs, graph=True)
+    with pytest.raises(SpmError) as ei:
+        p.autotune(F, outs, ignore_cache=True)
+    assert ei.value.status == -4
+    assert [p.info(n)["nblk"] for n in range(N)] == before
+    assert p.info()["device_bytes"] <= need + (64 << 10)
+    for graph in (False, True):
+        for o in outs:
+            o.fill_(float("nan"))
+        p.sweep(F, outs, graph=graph)
+        p.device_status()
+        for n in range(N):
+            want = O.mttkrp(c, v, dims, [f.cpu().numpy() for f in F], n)
+            assert O.relerr(outs[n].cpu().numpy(), want) <= 1e-5, (graph, n)
     p.close()
