@@ -408,7 +408,7 @@ int spmttkrp_plan_create(spmttkrp_plan_t* out, const int64_t* coo, const float* 
   // a default tile keeps two CTAs per SM (<= 110 KB each); a requested one is
   // only cut down to what one CTA can hold
   const size_t smem_cap = (o.tile ? 200 : 110) * 1024;
-  auto smem_of = [&](int t) { return mttkrp_smem_bytes(p->es, t, p->R, p->dtype, p->stages); };
+  auto smem_of = [&](int t) { return mttkrp_smem_bytes(p, t, p->stages); };
   while (p->tile > 32 && smem_of(p->tile) > smem_cap && smem_of(p->tile / 2) < smem_of(p->tile))
     p->tile /= 2;  // (a tile holds at least one chunk of each lane group)
   if (!p->host_only) {

@@ -550,7 +550,7 @@ int spmttkrp_autotune(spmttkrp_plan_t p, const void* const* factors, float* cons
     if (fixed_blocks && n > 48) continue;
     for (int t : {64, 128, 256})
       for (int sg : {2, 3})
-        if (mttkrp_smem_bytes(p->es, t, p->R, p->dtype, sg) <= 110 * 1024)
+        if (mttkrp_smem_bytes(p, t, sg) <= 110 * 1024)
           cands.push_back({n, t, 0, sg});
   }
   for (int n : {4, 8, 16, 32}) {

@@ -77,7 +77,7 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
   if (c.vec && c.VW == 4) {  // 8-byte lane slices: the FP32 kernel's lane shape
     switch (a.nmodes) {
       case 3:
-        if (c.L == 1) {  // one-lane groups: 32 runs per warp, 4 nonzeros of each per tile
+        if (warp_steps(a, c) == 4) {
           switch (a.mode + (a.es == 32 ? 0 : 3)) {
             case 0: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 0, 32>(a, c.L, s);
             case 1: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 1, 32>(a, c.L, s);
@@ -102,7 +102,7 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
       case 4: return launch_modes<4, __nv_bfloat16, 4, 4>(a, c.L, s);
       case 5: return launch_modes<5, __nv_bfloat16, 4, 4>(a, c.L, s);
       case 6: return launch_modes<6, __nv_bfloat16, 4, 4>(a, c.L, s);
-      default: return launch_warp_kernel<0, __nv_bfloat16, 4, 1, 4>(a, c.L, s);
+      default: return launch_any_modes<__nv_bfloat16, 4>(a, c, s);
     }
   }
   if (c.vec && c.VW == 8) {
@@ -128,9 +128,9 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
       default: return launch_warp_kernel<0, __nv_bfloat16, 8, 1, 4>(a, c.L, s);
     }
   }
-  if (c.vec) return launch_warp_kernel<0, __nv_bfloat16, 2, 1, 4>(a, c.L, s);
+  if (c.vec) return launch_any_modes<__nv_bfloat16, 2>(a, c, s);
   switch (c.RC) {
-    case 1: return launch_warp_kernel<0, __nv_bfloat16, 1, 1, 4>(a, c.L, s);
+    case 1: return launch_any_modes<__nv_bfloat16, 1>(a, c, s);
     case 2: return launch_warp_kernel<0, __nv_bfloat16, 1, 2, 4>(a, c.L, s);
     case 4: return launch_warp_kernel<0, __nv_bfloat16, 1, 4, 4>(a, c.L, s);
     default: return launch_warp_kernel<0, __nv_bfloat16, 1, 8, 2>(a, c.L, s);

@@ -50,13 +50,12 @@ int launch_mttkrp_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
     }
   }
   if (a.variant == 1) return launch_direct_float(a, c, s);
+  const int U = warp_steps(a, c);
   if (c.VW < 4 && narrow_built(a, c)) return launch_narrow_f32(a, c, s);
   if (c.vec && c.VW == 4) {
     switch (a.nmodes) {
       case 3:
-        // 4 in flight and 3 CTAs per SM when asked for, and for one-lane groups, whose
-        // warps hold 32 runs (their tiles hold 4 nonzeros per run)
-        if (a.es == 32 && (a.unroll == 4 || c.L == 1)) {
+        if (a.es == 32 && U == 4) {
           switch (a.mode) {
             case 0: return launch_warp_kernel<3, float, 4, 1, 4, 0, 32>(a, c.L, s);
             case 1: return launch_warp_kernel<3, float, 4, 1, 4, 1, 32>(a, c.L, s);
@@ -70,7 +69,7 @@ int launch_mttkrp_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
             default: return launch_warp_kernel<3, float, 4, 1, 8, 2, 32>(a, c.L, s);
           }
         }
-        if (a.unroll == 4 || c.L == 1) {
+        if (U == 4) {
           switch (a.mode) {
             case 0: return launch_warp_kernel<3, float, 4, 1, 4, 0, 16>(a, c.L, s);
             case 1: return launch_warp_kernel<3, float, 4, 1, 4, 1, 16>(a, c.L, s);
@@ -85,12 +84,12 @@ int launch_mttkrp_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
       case 4: return launch_modes<4, float, 4, 4>(a, c.L, s);
       case 5: return launch_modes<5, float, 4, 4>(a, c.L, s);
       case 6: return launch_modes<6, float, 4, 2>(a, c.L, s);
-      default: return launch_warp_kernel<0, float, 4, 1, 4>(a, c.L, s);
+      default: return launch_any_modes<float, 4>(a, c, s);
     }
   }
-  if (c.vec) return launch_warp_kernel<0, float, 2, 1, 4>(a, c.L, s);
+  if (c.vec) return launch_any_modes<float, 2>(a, c, s);
   switch (c.RC) {
-    case 1: return launch_warp_kernel<0, float, 1, 1, 4>(a, c.L, s);
+    case 1: return launch_any_modes<float, 1>(a, c, s);
     case 2: return launch_warp_kernel<0, float, 1, 2, 4>(a, c.L, s);
     case 4: return launch_warp_kernel<0, float, 1, 4, 4>(a, c.L, s);
     default: return launch_warp_kernel<0, float, 1, 8, 2>(a, c.L, s);

@@ -25,12 +25,13 @@ static LaneCfg cfg_for(const MttkrpArgs& a) {
   return warp_lane_config(a.R, a.dtype, fa, oa);
 }
 
-size_t mttkrp_smem_bytes(int es, int tile, int R, int dtype, int stages) {
+size_t mttkrp_smem_bytes(const spmttkrp_plan* p, int tile, int stages) {
   size_t m = 0;
-  for (size_t al : {16, 8, 4}) {
-    const LaneCfg c = warp_lane_config(R, dtype, al, al);
-    const int G = 32 / c.L;
-    m = std::max(m, (size_t)kWarps * warp_layout(es, warp_tile_for(tile, G, 4), stages, true).total);
+  for (size_t al : {16, 8, 4, 2}) {  // of the factors and the output, which come later
+    const LaneCfg c = warp_lane_config(p->R, p->dtype, al, al);
+    const int U = warp_steps(p->N, p->es, p->dtype, p->pack.packed, c, p->unroll);
+    const int tw = warp_tile_for(tile, 32 / c.L, U);
+    m = std::max(m, (size_t)kWarps * warp_layout(p->es, tw, stages, true).total);
   }
   return m;
 }

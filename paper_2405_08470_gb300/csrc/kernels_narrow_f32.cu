@@ -9,20 +9,26 @@
 
 namespace spm {
 
-template <int VW, int RC>
-static int launch_narrow(const MttkrpArgs& a, int L, cudaStream_t s) {
-  constexpr int NV = VW * RC;
+template <int VW, int RC, int U>
+static int launch_steps(const MttkrpArgs& a, int L, cudaStream_t s) {
   switch (a.nmodes) {
-    case 3: return launch_warp_kernel<3, float, VW, RC, 8>(a, L, s);
-    case 4: return launch_warp_kernel<4, float, VW, RC, 8>(a, L, s);
-    case 5: return launch_warp_kernel<5, float, VW, RC, NV == 1 ? 8 : 4>(a, L, s);
-    default: return launch_warp_kernel<6, float, VW, RC, NV == 1 ? 8 : 4>(a, L, s);
+    case 3: return launch_warp_kernel<3, float, VW, RC, U>(a, L, s);
+    case 4: return launch_warp_kernel<4, float, VW, RC, U>(a, L, s);
+    case 5: return launch_warp_kernel<5, float, VW, RC, VW * RC == 1 ? U : 4>(a, L, s);
+    default: return launch_warp_kernel<6, float, VW, RC, VW * RC == 1 ? U : 4>(a, L, s);
   }
 }
 
+template <int VW, int RC>
+static int launch_narrow(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
+  if constexpr (RC == 1)  // (only a one-piece row can have one-lane groups)
+    if (c.L == 1) return launch_steps<VW, RC, 4>(a, c.L, s);
+  return launch_steps<VW, RC, 8>(a, c.L, s);
+}
+
 int launch_narrow_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
-  if (c.VW == 2) return launch_narrow<2, 1>(a, c.L, s);
-  return c.RC == 1 ? launch_narrow<1, 1>(a, c.L, s) : launch_narrow<1, 2>(a, c.L, s);
+  if (c.VW == 2) return launch_narrow<2, 1>(a, c, s);
+  return c.RC == 1 ? launch_narrow<1, 1>(a, c, s) : launch_narrow<1, 2>(a, c, s);
 }
 
 }  // namespace spm

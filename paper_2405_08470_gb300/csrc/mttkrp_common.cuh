@@ -70,6 +70,34 @@ inline LaneCfg warp_lane_config(int R, int dtype, size_t factor_align, size_t ou
   return lane_config(R, dtype, false);
 }
 
+// Lanes of one or two values (ranks that are no multiple of four, or factors aligned
+// to less than 16 bytes): built for 3 to 6 modes and up to 64 columns; other shapes run
+// the runtime-modes kernel.
+inline bool narrow_built(int nmodes, bool packed, const LaneCfg& c) {
+  return nmodes >= 3 && nmodes <= 6 && !packed && c.VW * c.RC <= 2;
+}
+
+// Steps in flight (U) of the warp-block kernel for a shape: the dispatchers launch this many
+// and the plan sizes its tiles by it.  A tile holds at least one chunk of U G nonzeros, so
+// with one-lane groups (ranks 1, 2 and 4: G = 32) eight steps would stage 256 nonzeros: one
+// CTA per SM, and no room for a ring of 3 or 4 stages.  They take four (3M nonzeros, 3 modes,
+// rank 1, FP32: a sweep 0.235 ms, with eight 0.286), and two where a nonzero is wider than
+// 32 bytes (1.5M, 10 modes, rank 4: 0.90 ms, with four 1.07).
+inline int warp_steps(int nmodes, int es, int dtype, bool packed, const LaneCfg& c, int unroll) {
+  if (c.L == 1 && es > 32) return 2;
+  if (narrow_built(nmodes, packed, c)) {
+    if (c.L == 1) return 4;
+    return nmodes <= 4 || c.VW * c.RC == 1 ? 8 : 4;
+  }
+  if (c.VW == 8) return nmodes == 6 ? 2 : 4;
+  if (c.VW == 4) {
+    if (nmodes == 3)
+      return c.L == 1 || (unroll == 4 && dtype == SPM_DTYPE_F32) ? 4 : 8;
+    return nmodes == 6 && dtype == SPM_DTYPE_F32 ? 2 : 4;
+  }
+  return c.RC == 8 ? 2 : 4;
+}
+
 // ------------------------------------------------------------ stored nonzeros
 
 // Index k of a stored nonzeros (plain: word k; packed: its bit field).

@@ -1037,11 +1037,17 @@ int launch_modes(const MttkrpArgs& a, int L, cudaStream_t s) {
   return launch_warp_kernel<NT, T, VW, 1, U>(a, L, s);
 }
 
-// Lanes of one or two values (ranks that are no multiple of four, or factors aligned
-// to less than 16 bytes): built for 3 to 6 modes and up to 64 columns; other shapes run
-// the runtime-modes kernel.
 inline bool narrow_built(const MttkrpArgs& a, const LaneCfg& c) {
-  return a.nmodes >= 3 && a.nmodes <= 6 && !a.pk.packed && c.VW * c.RC <= 2;
+  return narrow_built(a.nmodes, a.pk.packed, c);
+}
+inline int warp_steps(const MttkrpArgs& a, const LaneCfg& c) {
+  return warp_steps(a.nmodes, a.es, a.dtype, a.pk.packed, c, a.unroll);
+}
+// The runtime-modes kernel with one- to four-value pieces (4 steps, or 2: warp_steps).
+template <typename T, int VW>
+int launch_any_modes(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
+  if (warp_steps(a, c) == 2) return launch_warp_kernel<0, T, VW, 1, 2>(a, c.L, s);
+  return launch_warp_kernel<0, T, VW, 1, 4>(a, c.L, s);
 }
 int launch_narrow_f32(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s);
 int launch_narrow_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s);
