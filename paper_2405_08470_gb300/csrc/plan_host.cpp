@@ -113,9 +113,10 @@ int default_nblk(int64_t nnz, int num_sms, int variant, bool capped) {
     const int64_t few = std::min<int64_t>(256, std::max<int64_t>(64, nnz / (sms * 8)));
     nb = std::max(std::min((nnz + few - 1) / few, sms * 128),
                   std::min((nnz + 511) / 512, sms * 1024));
-    // Under a memory cap at most 384 per SM, for the split rows' partials (2 R floats a
-    // block).
-    if (capped) nb = std::min(nb, sms * 384);
+    // Under a memory cap they hold 256 at least and there are at most 384 per SM: a block
+    // costs 2 R floats of partials, and a small plan cut into blocks of 64 needs 4 times
+    // the partials (78K nonzeros at rank 256: 2.5 MB against 0.6).
+    if (capped) nb = std::min((nnz + 255) / 256, sms * 384);
     nb = std::max(nb, (nnz + 4095) / 4096);
   } else if (variant == 2) {
     // tile form: about 16 blocks per SM, taken dynamically by the persistent
