@@ -181,41 +181,54 @@ __global__ void __launch_bounds__(256) gram_tile_kernel(const T* __restrict__ A,
 // the inverse, one symmetric sweep (Beaton's sweep operator) per pivot: with d = a_pp,
 //   a_ik -= a_ip a_kp / d,   a_ip = a_ip / d,   a_pp = -1 / d,
 // after which the matrix is -V^-1.  The pivots d are Cholesky's l_pp^2, so V is SPD
-// exactly when all of them are positive.  Thread (i, g) keeps row i's columns g, g + T,
-// .. in registers; only the pivot's column and 1 / d go through shared memory, written
-// by their owners a step ahead, so a step is one barrier.  What bounds it is the chain of
-// R divisions and barriers.  With the factorisation, substitution and product below in
-// shared memory (five barriers a column) it was most of a small tensor's iteration: three
-// iterations on 50K nonzeros at rank 16 took 0.97 ms, and take 0.52 with this, the Grams
-// of one chunk written directly and one block per row tile (60 us of it at rank 32).
+// exactly when all of them are positive.  The matrix lies in registers as 16 x 16 blocks,
+// one entry of each block on and below the diagonal per thread (the matrix stays
+// symmetric); only the pivot's column and 1 / d go through shared memory, written by their
+// owners a step ahead, so a step is one barrier.  What bounds it is the FP64 rate (two
+// multiply-adds per clock and SM) at R = 64 and the chain of R divisions and barriers below.
+// An ALS iteration on 20K nonzeros of 200 x 150 x 100 takes 0.127 / 0.201 / 0.411 / 0.503 ms
+// at rank 16 / 32 / 48 / 64.  With both halves of the matrix swept, a row's columns per
+// thread (16 products a step at rank 64 where these are 10), it took 0.130 / 0.252 / 0.611 /
+// 1.005, at rank 52 and above more than the factorisation, substitution and product below
+// in shared memory: 0.308 / 0.399 / 0.635 / 0.918.
 template <int RP>
 __global__ void __launch_bounds__(256) als_sweep_kernel(const double* __restrict__ grams, int N,
                                                         int n, int R, float* __restrict__ vinv,
                                                         int* __restrict__ status) {
-  constexpr int T = 256 / RP, Q = RP / T;  // threads per row, columns per thread
+  constexpr int B = RP / 16;      // blocks per side
   __shared__ double colp[2][RP];  // the pivot's column, double-buffered
   __shared__ double rdiag[2];     // 1 / pivot (0: not positive or not finite)
   __shared__ int bad;
-  const int tid = threadIdx.x, i = tid / T, g = tid % T;
+  const int tid = threadIdx.x, ti = tid / 16, tk = tid % 16;  // entry (ti, tk) of each block
   if (tid == 0) bad = *status;
   __syncthreads();
   if (bad) return;
-  double v[Q];
+  double v[B][B];  // blocks (a, b <= a): row ti + 16 a, column tk + 16 b
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int k = g + T * q;
-    v[q] = 1.0;
-    if (i < R && k < R)
-      for (int m = 0; m < N; ++m)
-        if (m != n) v[q] *= grams[(size_t)m * R * R + i * R + k];
-  }
-  // leaves column p (and the reciprocal of its pivot) for the next step
+  for (int a = 0; a < B; ++a)
+#pragma unroll
+    for (int b = 0; b <= a; ++b) {
+      const int i = ti + 16 * a, k = tk + 16 * b;
+      v[a][b] = 1.0;  // (entries past R take part in nothing that is used)
+      if (i < R && k < R)
+        for (int m = 0; m < N; ++m)
+          if (m != n) v[a][b] *= grams[(size_t)m * R * R + i * R + k];
+    }
+  // leaves column p (and the reciprocal of its pivot) for the next step: rows from p's
+  // block on lie in that column, the rows above it in row p
   auto publish = [&](int p) {
+    const int pb = p / 16, pe = p % 16;
+    double* col = colp[p & 1];
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
-      if (g + T * q == p && i < R) {
-        colp[p & 1][i] = v[q];
-        if (i == p) rdiag[p & 1] = v[q] > 0.0 && isfinite(v[q]) ? 1.0 / v[q] : 0.0;
+    for (int a = 0; a < B; ++a)
+#pragma unroll
+      for (int b = 0; b <= a; ++b) {
+        if (b == pb && tk == pe) {
+          col[ti + 16 * a] = v[a][b];
+          if (a == b && ti == pe)
+            rdiag[p & 1] = v[a][b] > 0.0 && isfinite(v[a][b]) ? 1.0 / v[a][b] : 0.0;
+        }
+        if (b < a && a == pb && ti == pe) col[tk + 16 * b] = v[a][b];
       }
   };
   publish(0);
@@ -226,21 +239,45 @@ __global__ void __launch_bounds__(256) als_sweep_kernel(const double* __restrict
       if (tid == 0) *status = SPM_ERR_NOT_SPD;
       return;
     }
-    const double ci = i < R ? colp[p & 1][i] : 0.0, si = ci * rd;
+    const int pb = p / 16, pe = p % 16;
+    const double* col = colp[p & 1];
+    double si[B], ck[B];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int k = g + T * q;
-      if (i < R && k < R) {
-        const double ck = colp[p & 1][k];
-        v[q] = i == p ? (k == p ? -rd : ck * rd) : (k == p ? si : fma(-si, ck, v[q]));
-      }
+    for (int a = 0; a < B; ++a) {
+      si[a] = col[ti + 16 * a] * rd;
+      ck[a] = col[tk + 16 * a];
+    }
+#pragma unroll
+    for (int a = 0; a < B; ++a)
+#pragma unroll
+      for (int b = 0; b <= a; ++b) v[a][b] = fma(-si[a], ck[b], v[a][b]);
+    if (tk == pe) {  // column p
+#pragma unroll
+      for (int a = 0; a < B; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b)
+          if (b == pb) v[a][b] = si[a];
+    }
+    if (ti == pe) {  // row p and the pivot
+#pragma unroll
+      for (int a = 0; a < B; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b)
+          if (a == pb) v[a][b] = a == b && tk == pe ? -rd : ck[b] * rd;
     }
     if (p + 1 < R) publish(p + 1);
     __syncthreads();
   }
 #pragma unroll
-  for (int q = 0; q < Q; ++q)
-    if (i < R && g + T * q < R) vinv[i * R + g + T * q] = (float)-v[q];
+  for (int a = 0; a < B; ++a)
+#pragma unroll
+    for (int b = 0; b <= a; ++b) {
+      const int i = ti + 16 * a, k = tk + 16 * b;
+      if (i < R && k < R) {
+        vinv[i * R + k] = (float)-v[a][b];
+        if (b < a) vinv[k * R + i] = (float)-v[a][b];
+      }
+    }
 }
 
 // R > 64: Cholesky, forward substitution and product in the global work buffer.  Every step is spread over the block, so no thread runs a long dependent chain:
