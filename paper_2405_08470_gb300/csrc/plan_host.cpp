@@ -101,17 +101,19 @@ int default_nblk(int64_t nnz, int num_sms, int variant, bool capped) {
   if (nnz <= 0) return 1;
   int64_t nb;
   if (variant == 0 || variant == 3) {
-    // warp blocks (forms 0 and 3), taken in order by the resident warps.  From 10M
-    // nonzeros on they hold 512 (the remap's stores then stay within what L2 holds: a
-    // 30M-nonzero sweep takes 2.28 ms with 512 and 2.37 with 1024; 256 pay more for
-    // their ends, 2.30), up to 1024 blocks per SM (larger blocks beyond: at 100M, 640
-    // and 1024 measure the same).  Below, 256, so that every warp has several to take,
-    // and on tensors too small for that fewer, down to 64, so that every SM has some (a
-    // sweep of 50K nonzeros takes 35 us with 64 and 47 with 256; of 200K, 52 with 192 and
-    // 60 with 256).
+    // warp blocks (forms 0 and 3), taken in order by the resident warps.  They hold 256
+    // while there are at most 384 per SM, so that every warp has several to take and no
+    // FP32 sum of a lane group is longer than that takes (12M nonzeros, 3 modes, rank 32:
+    // error against 64 bits 1.6e-7 and 0.89 ms a sweep; with 512, 1.95e-7 and 0.90; 20M, 6
+    // modes: 2.97 ms, with 512 2.93).  From there on they grow to 512 (the remap's stores
+    // then stay within what L2 holds: a 30M-nonzero sweep takes 2.28 ms with 512 and 2.37
+    // with 1024), up to 1024 blocks per SM (larger blocks beyond: at 100M, 640 and 1024
+    // measure the same).  On tensors too small for 256 they hold fewer, down to 64, so that
+    // every SM has some (a sweep of 50K nonzeros takes 35 us with 64 and 47 with 256; of
+    // 200K, 52 with 192 and 60 with 256).
     const int64_t sms = num_sms;
     const int64_t few = std::min<int64_t>(256, std::max<int64_t>(64, nnz / (sms * 8)));
-    nb = std::max(std::min((nnz + few - 1) / few, sms * 128),
+    nb = std::max(std::min((nnz + few - 1) / few, sms * 384),
                   std::min((nnz + 511) / 512, sms * 1024));
     // Under a memory cap they hold 256 at least and there are at most 384 per SM: a block
     // costs 2 R floats of partials, and a small plan cut into blocks of 64 needs 4 times

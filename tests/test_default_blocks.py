@@ -1,0 +1,42 @@
+"""Default block counts.  Every block costs 2 R floats of split-row partials, so a plan under a
+memory cap is cut into blocks of 256 nonzeros at least, at most 384 per SM and at most 4096
+nonzeros each, whatever an uncapped one would take."""
+import numpy as np
+import pytest
+
+from paper_2405_08470_gb300 import Plan
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("nnz", [1, 63, 64, 255, 256, 257, 1000, 50_000, 77_800, 311_000])
+def test_capped_plans_take_no_smaller_blocks(nnz):
+    dims = (1000, 997, 50)
+    k = np.arange(nnz, dtype=np.int64)
+    coo = np.stack([k % 1000, (k * 7 + k // 1000) % 997, k // 997 % 50], 1)
+    v = np.ones(nnz, np.float32)
+    p = Plan(coo, v, dims, 8, host_only=True, max_bytes=1 << 40)
+    sms = p.info()["num_sms"]
+    want = max(min(sms * 384, -(-nnz // 256)), -(-nnz // 4096))
+    for n in range(3):
+        assert p.info(n)["nblk"] == want, n
+    p.close()
+
+
+@pytest.mark.parametrize("nnz", [11_000_001, 14_600_000])
+def test_blocks_hold_256_nonzeros_while_they_are_few(nnz):
+    """A block's lane groups each add their share of its nonzeros in FP32, so longer blocks
+    round more: up to 384 blocks per SM they hold 256."""
+    dims = (5000, 4001)
+    k = np.arange(nnz, dtype=np.int64)
+    p = Plan(np.stack([k // 4001, k % 4001], 1), np.ones(nnz, np.float32), dims, 8, host_only=True)
+    sms = p.info()["num_sms"]
+    want = max(min(sms * 384, -(-nnz // 256)), min(sms * 1024, -(-nnz // 512)))
+    for n in range(2):
+        assert p.info(n)["nblk"] == want
+        assert np.diff(p.bounds(n)).max() <= 257
+    p.close()
