@@ -311,7 +311,8 @@ enum {
                          partition, bit7 nonzeros carry their remap ids, bits 8-9
                          variant, bit10 nonzeros carry write orders, bits 11-31
                          hot rows per factor, 0 = no hot-row flags), SMs,
-                         |X|^2 (double), lanes                                      */
+                         |X|^2 (double), lanes per nonzero of the plan's kernel form
+                         (16-byte aligned factors)                                  */
   SPM_Q_NEXT_POS = 1, /* int32[nnz]: next_pos of `mode`                            */
   SPM_Q_BOUNDS = 2,   /* int64[nblk+1]: block boundaries of `mode`                 */
   SPM_Q_SPLITS = 3,   /* int64[nsplit][3]: (row, first_blk, last_blk) of `mode`   */

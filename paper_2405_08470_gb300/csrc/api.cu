@@ -685,7 +685,7 @@ int spmttkrp_plan_query(spmttkrp_plan_t p, int what, int mode, void* dst, size_t
       o[12] = p->host_only;
       o[13] = p->num_sms;
       std::memcpy(&o[14], &p->normx2, 8);
-      o[15] = lane_config(p->R, p->dtype, true).L;
+      o[15] = plan_lanes(p);
       o[12] = (int64_t)p->host_only | ((int64_t)(p->variant & 1) << 1) |
               ((int64_t)p->keep_base << 2) | ((int64_t)p->stages << 3) |
               ((int64_t)p->partition << 6) | ((int64_t)p->alpha << 7) |

@@ -25,6 +25,11 @@ static LaneCfg cfg_for(const MttkrpArgs& a) {
   return warp_lane_config(a.R, a.dtype, fa, oa);
 }
 
+int plan_lanes(const spmttkrp_plan* p) {
+  return (p->variant == 1 || p->variant == 2 ? lane_config(p->R, p->dtype, true)
+                                             : warp_lane_config(p->R, p->dtype, 16, 16)).L;
+}
+
 size_t mttkrp_smem_bytes(const spmttkrp_plan* p, int tile, int stages) {
   size_t m = 0;
   for (size_t al : {16, 8, 4, 2}) {  // of the factors and the output, which come later

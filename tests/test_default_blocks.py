@@ -40,3 +40,17 @@ def test_blocks_hold_256_nonzeros_while_they_are_few(nnz):
         assert p.info(n)["nblk"] == want
         assert np.diff(p.bounds(n)).max() <= 257
     p.close()
+
+
+@pytest.mark.parametrize("R,dtype,variant,lanes", [
+    (10, "f32", 0, 8), (10, "f32", 3, 8), (25, "f32", 0, 32), (32, "f32", 0, 8), (50, "f32", 0, 32),
+    (32, "bf16", 0, 8), (64, "bf16", 0, 8), (36, "bf16", 0, 16), (10, "f32", 1, 16),
+    (32, "bf16", 1, 4), (32, "f32", 2, 8)])
+def test_plan_reports_the_lanes_of_its_kernel_form(R, dtype, variant, lanes):
+    # forms 0 and 3: the widest piece of at most 16 bytes (8 for BF16 rows of at most 32
+    # values) that divides the rank, lanes rounded up to a power of two; forms 1 and 2:
+    # 16-byte pieces or single values
+    coo = np.stack([np.arange(50), np.arange(50) % 7, np.arange(50) % 5], 1).astype(np.int64)
+    p = Plan(coo, np.ones(50, np.float32), (50, 7, 5), R, dtype=dtype, variant=variant, host_only=True)
+    assert p.info()["lanes"] == lanes
+    p.close()
