@@ -401,16 +401,17 @@ int spmttkrp_plan_create(spmttkrp_plan_t* out, const int64_t* coo, const float* 
   // 3-mode nonzeros in 32-byte sectors carry their remap ids in the padding (the
   // element tuple of Section 3.5), so the fused pass reads no next_pos array
   p->alpha = (nmodes == 3 && p->es == 32) ? 1 : 0;
-  // ring depth: 2 stages for 32-byte and wider nonzeros (a tile of 128 of
-  // them is 4 KB, so two in flight keep the copies ahead), 3 for 16-byte ones
+  // ring depth: 2 stages for 32-byte and wider nonzeros, 3 for 16-byte ones (a tile of
+  // either is 2 KB by default)
   if (!p->stages) p->stages = p->es >= 32 ? 2 : 3;
   p->tile = o.tile ? o.tile : default_tile(p->es);
-  // a default tile keeps two CTAs per SM (<= 110 KB each); a requested one is
-  // only cut down to what one CTA can hold
+  // a default tile is cut until two CTAs fit an SM (<= 110 KB each), a requested one to
+  // what one CTA can hold, but never below a chunk of the lane groups; the steps of a
+  // chunk are chosen so that both hold (warp_steps)
   const size_t smem_cap = (o.tile ? 200 : 110) * 1024;
   auto smem_of = [&](int t) { return mttkrp_smem_bytes(p, t, p->stages); };
   while (p->tile > 32 && smem_of(p->tile) > smem_cap && smem_of(p->tile / 2) < smem_of(p->tile))
-    p->tile /= 2;  // (a tile holds at least one chunk of each lane group)
+    p->tile /= 2;
   if (!p->host_only) {
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess)
@@ -443,7 +444,7 @@ int spmttkrp_plan_create(spmttkrp_plan_t* out, const int64_t* coo, const float* 
     st = plan_dalloc(p, (void**)&p->d_elem[0], eb);
     if (!st) st = plan_dalloc(p, (void**)&p->d_elem[1], eb);
     if (!st && p->keep_base) st = plan_dalloc(p, (void**)&p->d_base, eb);
-    // d_err[0]: device error word; d_err[1]: the tile form's block counter
+    // d_err[0]: device error word; d_err[1]: the counter of claimed blocks
     if (!st) st = plan_dalloc(p, (void**)&p->d_err, 4 * sizeof(int));
     if (!st) {
       cudaError_t e = cudaMemsetAsync(p->d_err, 0, 4 * sizeof(int), p->stream);

@@ -49,9 +49,10 @@ constexpr int kFixChunk = 256;  // blocks summed by one CTA of the fix-up's firs
 
 // Empty output rows (forms 0 and 3) come from a list of their runs, in pieces of at most
 // kGapRows rows that all lane groups of the fused kernel share.  Zeroed by whoever wrote
-// the next nonempty row, as the other forms do, an unused range of 180K ids held one mode
+// the next nonempty row, as the other forms do, an unused range of 131K ids held one mode
 // of a 20M-nonzero 5-mode tensor for 3.3 ms (0.65 of them for its nonzeros), and the code
-// for it stood in every place where a row can end.
+// for it stood in every place where a row can end.  (That tensor's generator leaves the
+// range unused: its coordinates come from keys that wrap past 2^63.)
 constexpr int kGapRows = 64;
 
 // Host-side result of planning one mode.
@@ -142,7 +143,7 @@ struct spmttkrp_plan {
   std::vector<spm::ModeDev> md;
   float* d_part = nullptr;   // split-row partials: max nblk x 2 x R
   size_t part_cap = 0;       // floats
-  int* d_err = nullptr;      // device error word [0] and the tile form's block counter [1]
+  int* d_err = nullptr;      // device error word [0] and the counter of claimed blocks [1]
   // ALS / CP-loss scratch (allocated on first use)
   float* d_M = nullptr;       // max_n dims[n] x R: spMTTKRP output of the ALS mode
   float* d_U = nullptr;       // max_n dims[n] x R: M V^-1 before normalisation (R > 64)
@@ -255,7 +256,8 @@ struct MttkrpArgs {
                            // nothing completes, so it gives up after wait_ns
   int64_t nnz;             // nonzeros of the working copy (form 2 stages whole tiles)
   int grid_ctas;           // form 2: persistent CTAs (0 = one per block)
-  int* sched;              // form 2: device block counter (zeroed by the launcher)
+  int* sched;              // device counter of claimed blocks (forms 0 and 2; zeroed by the
+                           // launcher where blocks are claimed)
   PackInfo pk;             // index layout of the stored nonzeros
   double* loss_part;       // fused CP-loss pass: one FP64 partial of sum e^2 per block
                            // (non-null selects the fused pass: see mttkrp_warp_kernel)

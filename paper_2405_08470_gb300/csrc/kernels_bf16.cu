@@ -77,7 +77,7 @@ int launch_mttkrp_bf16(const MttkrpArgs& a, const LaneCfg& c, cudaStream_t s) {
   if (c.vec && c.VW == 4) {  // 8-byte lane slices: the FP32 kernel's lane shape
     switch (a.nmodes) {
       case 3:
-        if (warp_steps(a, c) == 4) {
+        if (warp_steps(a, c) == 4) {  // one-lane groups
           switch (a.mode + (a.es == 32 ? 0 : 3)) {
             case 0: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 0, 32>(a, c.L, s);
             case 1: return launch_warp_kernel<3, __nv_bfloat16, 4, 1, 4, 1, 32>(a, c.L, s);

@@ -151,16 +151,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
-// 16-byte asynchronous copy global -> shared by one thread, and the wait for all of
-// the thread's copies.
-__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
 // 1D bulk async copy with an L2 cache policy (e.g. evict_first for streams).
 __device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32_t bytes,
                                               uint64_t* bar, uint64_t policy) {
@@ -306,15 +296,6 @@ struct Slice<float, 4> {
     x[2] = v.z;
     x[3] = v.w;
   }
-  __device__ __forceinline__ static void load_hint(const void* base, int64_t row, int R, int sub,
-                                                   uint64_t pol, float* x) {
-    const uint4 v = ld_nc_hint_v4(
-        reinterpret_cast<const float4*>(static_cast<const float*>(base) + row * R) + sub, pol);
-    x[0] = __uint_as_float(v.x);
-    x[1] = __uint_as_float(v.y);
-    x[2] = __uint_as_float(v.z);
-    x[3] = __uint_as_float(v.w);
-  }
 };
 
 template <>
@@ -331,14 +312,6 @@ struct Slice<__nv_bfloat16, 8> {
                                               float* x) {
     unpack(__ldg(reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(base) + row * R) +
                  sub),
-           x);
-  }
-  __device__ __forceinline__ static void load_hint(const void* base, int64_t row, int R, int sub,
-                                                   uint64_t pol, float* x) {
-    unpack(ld_nc_hint_v4(
-               reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(base) + row * R) +
-                   sub,
-               pol),
            x);
   }
 };

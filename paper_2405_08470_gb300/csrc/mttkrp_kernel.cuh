@@ -50,7 +50,6 @@
 
 namespace spm {
 
-constexpr int kMaxStages = 4;  // tiles per warp ring: stages - 1 in flight while one is used
 constexpr int kWarps = kThreads / 32;
 
 // Per-warp shared-memory layout (bytes, in order): the staged tiles, their remap
@@ -326,14 +325,14 @@ __device__ __forceinline__ void store_piece(float* __restrict__ d, const float* 
 // CTAs per SM the register budget is cut for.  Wide lanes (16 bytes of every
 // gathered row in flight) take 128 registers and two CTAs; lanes that hold at most 24
 // registers in flight take three.
-template <int NT, int VW, int RC, int U, bool LOSS>
+template <int NT, int VW, int RC, int U>
 constexpr int warp_min_ctas() {
   return NT > 0 && VW * RC <= 2 && U * (NT - 1) * VW * RC <= 24 ? 3 : 2;
 }
 
 template <int NT, typename T, int VW, int RC, int U, int MODE, int ESB = 0, bool LOSS = false,
           bool RWARP = false, bool PK = false>
-__global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>()))
+__global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U>()))
     mttkrp_warp_kernel(const MttkrpArgs a, const int L) {
   static_assert(!LOSS || (NT == 3 && MODE >= 0 && VW > 1 && U == 4 && (ESB == 32 || ESB == 16)),
                 "the fused CP-loss pass is built for 3 modes and 16- or 32-byte nonzeros");
@@ -363,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
       return;
     }
   }
-  const int nwarps = gridDim.x * CW;  // blocks w, w + nwarps, ... belong to warp w
+  const int nwarps = gridDim.x * CW;  // blocks w and w + nwarps are warp w's, then claimed ones
 
   extern __shared__ __align__(128) uint8_t smem[];
   uint8_t* wbase = smem + (size_t)warp * lay.total;
@@ -384,9 +383,9 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
 
   // ---- staging.  Lane 0 walks the warp's blocks tile by tile, one stage each: a
-  // descriptor {first position, nonzeros | flags << 16, block, 0}, then one mbarrier arrival with the tile's byte count.  A tile of no
-  // nonzeros ends the sequence.
-  constexpr int kFirst = 4, kLast = 8;  // tile flags beside BLK_HEAD_SPLIT, BLK_TAIL_SPLIT
+  // descriptor {first position, nonzeros | flags << 16, block, 0}, then one mbarrier arrival
+  // with the tile's byte count.  A tile of no nonzeros ends the sequence.
+  constexpr int kLast = 4;  // the block's last tile (beside BLK_HEAD_SPLIT, BLK_TAIL_SPLIT)
   int in_flight = 0;                    // tiles issued and not yet waited for
   // lane 0: block and position, the next block and its descriptor, the one after
   int ib = 0, ipos = 0, ihi = 0, ib1 = blockIdx.x * CW + warp, ib2 = ib1 + nwarps;
@@ -411,8 +410,8 @@ __global__ void __launch_bounds__(kThreads, (warp_min_ctas<NT, VW, RC, U, LOSS>(
         if (LOSS && ipos >= ihi) a.loss_part[ib] = 0.0;
       }
       const int n = ipos < ihi ? min(TW, ihi - ipos) : 0;
-      const int fl = ibi.w | (ipos == ibi.x ? kFirst : 0) | (ipos + n == ihi ? kLast : 0);
-      desc[st] = make_int4(ipos, n | (fl << 16), ib, ibi.z);
+      const int fl = ibi.w | (ipos + n == ihi ? kLast : 0);
+      desc[st] = make_int4(ipos, n | (fl << 16), ib, 0);
       const uint32_t ebytes = (uint32_t)n * es;
       uint32_t npbytes = 0;
       const int np0 = ipos & ~3;
