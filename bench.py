@@ -777,7 +777,7 @@ def main():
     t_roof_ms = sum(byts) / (peak * 1e9) * 1e3
     achieved = sum(byts) / (per_mode.sum() * 1e-3) / 1e9
     traffic = ncu_traffic(args.workload, R, args.dtype, nnz,
-                          dict(info, unroll=args.unroll or 8, cache_hints=args.hints,
+                          dict(info, unroll=info["steps"], cache_hints=args.hints,
                                blocks_per_sm=info["nblk"] / info["num_sms"]))
     # per-nonzero gathers counted every time (no reuse in L1/L2), for comparison
     E = 4 * N + 4
@@ -878,7 +878,7 @@ def main():
                                        "warp blocks, bulk-async staged tiles, one remap warp "
                                        "per CTA storing in destination order"][info["variant"]],
                        "autotuned": bool(args.autotune),
-                       "unroll": args.unroll or 8, "cache_hints": args.hints,
+                       "unroll": info["steps"], "cache_hints": args.hints,
                        "stages": info["stages"],
                        "element_bytes": info["elem_bytes"],
                        "keep_base": bool(args.keep_base),

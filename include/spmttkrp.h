@@ -88,7 +88,10 @@ typedef struct {
                        0; otherwise form 0 runs): 7 warps per CTA compute and
                        the 8th stores the CTA's 960-nonzero write-order tiles
                        in destination order                                     */
-  int unroll;       /* steps in flight per lane group in form 0, 3 modes: 0 (= 8), 4, 8 */
+  int unroll;       /* steps in flight per lane group in form 0: 0 (= 8), 4 or 8 for FP32
+                       with 3 modes, 16-byte lanes and more than 4 columns; every
+                       other shape runs a fixed number of 2, 4 or 8 (the info query
+                       reports it)                                              */
   int stages;       /* tiles per warp ring in form 0: 0 (= 2 for 32-byte and wider
                        nonzeros, 3 for 16-byte ones), 2, 3 or 4                   */
   int element_bytes;/* stride of a stored nonzero (N int32 indices + FP32 value):
@@ -310,7 +313,8 @@ enum {
                          variant & 1, bit2 keep_base, bits 3-5 ring stages, bit6
                          partition, bit7 nonzeros carry their remap ids, bits 8-9
                          variant, bit10 nonzeros carry write orders, bits 11-31
-                         hot rows per factor, 0 = no hot-row flags), SMs,
+                         hot rows per factor, 0 = no hot-row flags, bits 32-35
+                         steps in flight of form 0), SMs,
                          |X|^2 (double), lanes per nonzero of the plan's kernel form
                          (16-byte aligned factors)                                  */
   SPM_Q_NEXT_POS = 1, /* int32[nnz]: next_pos of `mode`                            */

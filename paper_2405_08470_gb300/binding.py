@@ -364,6 +364,7 @@ class Plan:
         d["host_only"], d["variant"], d["keep_base"] = flags & 1, (flags >> 8) & 3, (flags >> 2) & 1
         d["write_orders"] = (flags >> 10) & 1
         d["hot_rows"] = (flags >> 11) & 0x1FFFFF
+        d["steps"] = (flags >> 32) & 15
         d["stages"] = (flags >> 3) & 7
         d["partition"] = (flags >> 6) & 1
         d["remap_ids_in_elements"] = (flags >> 7) & 1

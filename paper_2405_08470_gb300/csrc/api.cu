@@ -691,7 +691,7 @@ int spmttkrp_plan_query(spmttkrp_plan_t p, int what, int mode, void* dst, size_t
               ((int64_t)p->keep_base << 2) | ((int64_t)p->stages << 3) |
               ((int64_t)p->partition << 6) | ((int64_t)p->alpha << 7) |
               ((int64_t)p->variant << 8) | ((int64_t)p->worders << 10) |
-              ((int64_t)p->hot_rows << 11);
+              ((int64_t)p->hot_rows << 11) | ((int64_t)plan_steps(p) << 32);
       return SPM_OK;
     }
     case SPM_Q_NEXT_POS: {

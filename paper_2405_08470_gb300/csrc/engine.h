@@ -282,8 +282,10 @@ int launch_loss_reduce(const double* part, int64_t n, float* loss, double* loss6
 // remap-only pass in destination order (plans with write orders): mode -> mode+1
 int launch_remap_ordered(const uint8_t* in, uint8_t* out, int64_t nnz, int mode, int* err,
                          cudaStream_t s);
-// Lanes per nonzero of the plan's kernel form, for 16-byte aligned factors and output.
+// Lanes per nonzero of the plan's kernel form, and steps in flight of the warp-block form,
+// for 16-byte aligned factors and output.
 int plan_lanes(const spmttkrp_plan* p);
+int plan_steps(const spmttkrp_plan* p);
 // Dynamic shared memory of a form-0 CTA with this tile and ring, for the factor alignment
 // that needs most.
 size_t mttkrp_smem_bytes(const spmttkrp_plan* p, int tile, int stages);

@@ -30,6 +30,11 @@ int plan_lanes(const spmttkrp_plan* p) {
                                              : warp_lane_config(p->R, p->dtype, 16, 16)).L;
 }
 
+int plan_steps(const spmttkrp_plan* p) {
+  return warp_steps(p->N, p->es, p->dtype, p->pack.packed, warp_lane_config(p->R, p->dtype, 16, 16),
+                    p->unroll);
+}
+
 size_t mttkrp_smem_bytes(const spmttkrp_plan* p, int tile, int stages) {
   size_t m = 0;
   for (size_t al : {16, 8, 4, 2}) {  // of the factors and the output, which come later

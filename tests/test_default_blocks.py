@@ -54,3 +54,18 @@ def test_plan_reports_the_lanes_of_its_kernel_form(R, dtype, variant, lanes):
     p = Plan(coo, np.ones(50, np.float32), (50, 7, 5), R, dtype=dtype, variant=variant, host_only=True)
     assert p.info()["lanes"] == lanes
     p.close()
+
+
+@pytest.mark.parametrize("N,R,dtype,unroll,element_bytes,steps", [
+    (3, 32, "f32", 0, 0, 8), (3, 32, "f32", 4, 0, 4), (3, 32, "f32", 8, 16, 8), (3, 4, "f32", 8, 0, 4),
+    (3, 25, "f32", 4, 0, 8), (3, 32, "bf16", 4, 0, 8), (3, 64, "bf16", 8, 0, 4), (3, 2, "f32", 0, 0, 4),
+    (4, 32, "f32", 8, 0, 4), (5, 50, "f32", 0, 0, 4), (6, 32, "f32", 0, 0, 2), (6, 32, "bf16", 0, 0, 4),
+    (7, 1, "f32", 0, 0, 4), (8, 1, "f32", 0, 0, 2), (2, 32, "f32", 0, 0, 4)])
+def test_plan_reports_its_steps_in_flight(N, R, dtype, unroll, element_bytes, steps):
+    # the unroll option is for FP32 with 3 modes and 16-byte lanes; elsewhere it is fixed
+    coo = np.stack([np.arange(50) % (50 - n) for n in range(N)], 1).astype(np.int64)
+    p = Plan(coo, np.ones(50, np.float32), [50 - n for n in range(N)], R, dtype=dtype,
+             unroll=unroll, element_bytes=element_bytes, host_only=True)
+    assert p.info()["steps"] == steps
+    assert p.info()["hot_rows"] == 0 and p.info()["host_only"] == 1
+    p.close()
