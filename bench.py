@@ -199,7 +199,7 @@ def kernel_digest():
 
 def ncu_traffic(workload, R, dtype, nnz, info):
     """DRAM bytes per launch of the fused kernel from a committed ncu summary: bytes
-    measured on a smaller tensor of the same shape (one kernel, its three mode
+    measured on a tensor of the same shape (one kernel, its three mode
     launches), scaled to this run's nonzero count (per-nonzero traffic: the stream,
     the scattered copy and the factor-row misses all grow with the nonzeros).
     Used only while the kernel sources hash to the captured digest and the run has
@@ -214,13 +214,11 @@ def ncu_traffic(workload, R, dtype, nnz, info):
         return None
     if d.get("kernel_digest") != kernel_digest():
         return None
-    e = d.get("entries", {}).get(f"{workload}_R{R}_{dtype}")
-    if not e:
-        return None
-    cfg = e.get("config", {})
-    if any(info.get(k) != v for k, v in cfg.items()):
-        return None
-    return e["dram_bytes_per_nonzero_per_launch"] * nnz
+    e = d.get("entries", {}).get(f"{workload}_R{R}_{dtype}", {})
+    for c in (e, *e.get("other_configurations", [])):
+        if c and all(info.get(k) == v for k, v in c["config"].items()):
+            return c["dram_bytes_per_nonzero_per_launch"] * nnz
+    return None
 
 
 def cpu_oracle_full(coo_h, vals_h, dims, R, seed, one_thread_seconds=4.0):
